@@ -213,6 +213,119 @@ LWE_DEV uint4 aes_ctr_run_block(const AesTab &tab, const uint32_t rk[44], const 
   return make_uint4(o0 ^ rk[40], o1 ^ rk[41], o2 ^ rk[42], o3 ^ rk[43]);
 }
 
+// Counter blocks at arbitrary indices below 2^32, under one key: the first
+// two rounds as table entries.  The index enters as s3 = bswap32(index) and,
+// after ShiftRows, index byte j (j = 0 the lowest) reaches column j of round
+// 1 alone.  So every column of round 2 is the XOR of four terms, each a
+// function of one index byte; F_j holds the four terms of byte j, F_3 with
+// round key 2.  Two rounds then cost two 16-byte loads (F_0 and F_1; F_2 ^
+// F_3 changes every 65536 blocks and stays in registers) instead of 32
+// lookups, for any order of the blocks, where aes_ctr_run needs consecutive
+// ones: the products visit blocks n / 8 apart.
+#define AES_F_ENTRIES (3 * 256)              // F_0, F_1, F_2
+#define AES_F_BYTES (AES_F_ENTRIES * 16)     // 12 KB
+
+// entry x of F_J; rk may be in shared memory
+template <int J>
+LWE_DEV uint4 aes_f_entry(const AesTab &tab, const uint32_t *rk, uint64_t domain, uint32_t x) {
+  const uint32_t s0 = bswap32((uint32_t)(domain >> 32)) ^ rk[0];
+  const uint32_t s1 = bswap32((uint32_t)domain) ^ rk[1];
+  const uint32_t s2 = rk[2], s3 = rk[3] ^ (x << (8 * (3 - J)));
+  if (J == 0) {
+    const uint32_t t = tab.T<0, 0>(s0) ^ tab.T<1, 1>(s1) ^ tab.T<2, 2>(s2) ^ tab.T<3, 3>(s3) ^ rk[4];
+    return make_uint4(tab.T<0, 0>(t), tab.T<3, 3>(t), tab.T<2, 2>(t), tab.T<1, 1>(t));
+  }
+  if (J == 1) {
+    const uint32_t t = tab.T<0, 0>(s1) ^ tab.T<1, 1>(s2) ^ tab.T<2, 2>(s3) ^ tab.T<3, 3>(s0) ^ rk[5];
+    return make_uint4(tab.T<1, 1>(t), tab.T<0, 0>(t), tab.T<3, 3>(t), tab.T<2, 2>(t));
+  }
+  if (J == 2) {
+    const uint32_t t = tab.T<0, 0>(s2) ^ tab.T<1, 1>(s3) ^ tab.T<2, 2>(s0) ^ tab.T<3, 3>(s1) ^ rk[6];
+    return make_uint4(tab.T<2, 2>(t), tab.T<1, 1>(t), tab.T<0, 0>(t), tab.T<3, 3>(t));
+  }
+  const uint32_t t = tab.T<0, 0>(s3) ^ tab.T<1, 1>(s0) ^ tab.T<2, 2>(s1) ^ tab.T<3, 3>(s2) ^ rk[7];
+  return make_uint4(tab.T<3, 3>(t) ^ rk[8], tab.T<2, 2>(t) ^ rk[9], tab.T<1, 1>(t) ^ rk[10],
+                    tab.T<0, 0>(t) ^ rk[11]);
+}
+
+// Where entry x of F_1 sits: lanes that hold rows of A read entries n / 2048
+// apart per row, which for a large power of two would be one bank group.
+LWE_DEV uint32_t aes_f1_at(uint32_t x) { return 256 + (x ^ (((x >> 3) ^ (x >> 6)) & 7u)); }
+
+// F_0 .. F_2 of one key and stream, by threads t, t + nt, ... (the caller
+// synchronises before they are read)
+LWE_DEV void aes_f_fill(uint4 *f, const AesTab &tab, const uint32_t *rk, uint64_t domain,
+                        uint32_t t, uint32_t nt) {
+  for (uint32_t x = t; x < AES_F_ENTRIES; x += nt) {
+    const uint32_t b = x & 255u;
+    f[x >= 256 && x < 512 ? aes_f1_at(b) : x] =
+        x < 256 ? aes_f_entry<0>(tab, rk, domain, b)
+                : (x < 512 ? aes_f_entry<1>(tab, rk, domain, b)
+                           : aes_f_entry<2>(tab, rk, domain, b));
+  }
+}
+
+struct AesF {
+  const uint4 *f;      // F_0, F_1, F_2 in shared memory
+  const uint32_t *rk;  // the key's round keys in shared memory
+  uint32_t cur;        // index >> 16 of f23
+  uint32_t f23[4];     // F_2 ^ F_3 there
+};
+
+LWE_DEV AesF aes_f_open(const uint4 *f, const uint32_t *rk) {
+  AesF a;
+  a.f = f;
+  a.rk = rk;
+  a.cur = ~0u;
+  a.f23[0] = a.f23[1] = a.f23[2] = a.f23[3] = 0;
+  return a;
+}
+
+// State after round 2 of block `index` of stream `domain`.
+LWE_DEV void aes_f_start(AesF &a, const AesTab &tab, uint64_t domain, uint32_t index,
+                         uint32_t s[4]) {
+  if ((index >> 16) != a.cur) {  // every 65536 blocks
+    a.cur = index >> 16;
+    const uint4 w = aes_f_entry<3>(tab, a.rk, domain, a.cur >> 8), v = a.f[512 + (a.cur & 255u)];
+    a.f23[0] = v.x ^ w.x;
+    a.f23[1] = v.y ^ w.y;
+    a.f23[2] = v.z ^ w.z;
+    a.f23[3] = v.w ^ w.w;
+  }
+  const uint4 u = a.f[index & 255u], v = a.f[aes_f1_at((index >> 8) & 255u)];
+  s[0] = u.x ^ v.x ^ a.f23[0];
+  s[1] = u.y ^ v.y ^ a.f23[1];
+  s[2] = u.z ^ v.z ^ a.f23[2];
+  s[3] = u.w ^ v.w ^ a.f23[3];
+}
+
+// Rounds 3 .. 9 of NB blocks side by side (independent lookups in flight).
+// rk: round keys 12 .. 39 of the key schedule.
+template <int NB>
+LWE_DEV void aes_rounds_3_9(const AesTab &tab, const uint32_t rk[28], uint32_t s[NB][4]) {
+#pragma unroll
+  for (int r = 0; r < 7; r++) {
+#pragma unroll
+    for (int b = 0; b < NB; b++) {
+      uint32_t t[4];
+#pragma unroll
+      for (int c = 0; c < 4; c++)
+        t[c] = tab.T<0, 0>(s[b][c]) ^ tab.T<1, 1>(s[b][(c + 1) & 3]) ^
+               tab.T<2, 2>(s[b][(c + 2) & 3]) ^ tab.T<3, 3>(s[b][(c + 3) & 3]) ^ rk[4 * r + c];
+#pragma unroll
+      for (int c = 0; c < 4; c++) s[b][c] = t[c];
+    }
+  }
+}
+
+// The last round's SubBytes with the bytes gathered as a kernel multiplies
+// them: S(byte B0 of w0) in byte 0 and S(byte B1 of w1) in byte 2 (T3 and T1
+// hold S there), XOR k.
+template <int B0, int B1>
+LWE_DEV uint32_t aes_last2(const AesTab &tab, uint32_t w0, uint32_t w1, uint32_t k) {
+  return ((tab.T<3, B0>(w0) & 0x000000ffu) ^ k) ^ (tab.T<1, B1>(w1) & 0x00ff0000u);
+}
+
 // Load a 16-byte key from memory as four little-endian words.
 LWE_DEV void aes_load_key(const uint8_t *key, uint32_t k[4]) {
   if ((reinterpret_cast<uintptr_t>(key) & 15) == 0) {

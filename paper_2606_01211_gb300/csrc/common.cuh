@@ -16,7 +16,6 @@ enum LweKernel {
   KID_DECRYPT,
   KID_MUL_SA,
   KID_MUL_SA_FUSED,
-  KID_V_ENCODE,
   KID_TREE,
   KID_FINAL_KEY,
   KID_DERIVE,

@@ -1,20 +1,20 @@
-// kem_kernels.cu -- CUDA-core kernels of the plain-LWE KEM hot path (sm_103a).
+// kem_kernels.cu -- kernels of the plain-LWE KEM hot path (sm_103a) but for
+// the batched GEMM (gemm_tc.cu).
 //
 //   k_expand_A      sample(seedA) of Alg. 1: AES-128-CTR expansion of A,
 //                   16-byte coalesced stores.
 //   k_noise         the error/secret distributions of Alg. 1-2 (Tab. 1:
 //                   rounded Gaussian) by CDF-table inverse sampling of AES
 //                   counter streams.
-//   k_mul_as_rows, k_mul_as_fused: B = A S + E of Alg. 1 (A stored, or
-//                   regenerated from its seed in-CTA).
+//   products.cuh    k_mul_as, k_mul_as_gen, k_mul_as_gen_split: B = A S + E
+//                   of Alg. 1 (A stored, or regenerated from its seed);
+//                   k_sa, k_sa_gen: B' = S' A + E' and C = S' B + E'' +
+//                   Enc(mu) of Alg. 2, with a compare epilogue for Alg. 5.
 //   k_decrypt       M = C - B' S and mu' = Dec(M) of Alg. 3.
-//   k_sa            B' = S' A + E' of Alg. 2 on the CUDA cores (A stored or
-//                   regenerated from its seed in-CTA), with a compare
-//                   epilogue for Alg. 5.
-//   k_v_encode      V = S' B + E'', C = V + Enc(mu) of Alg. 2 (or compare).
 //   k_keygen_seeds, k_derive, k_tree, k_final_key: the hashing of
 //                   Alg. 4-5 (SHA3-256) and the Fujisaki-Okamoto selection.
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 
 #include <algorithm>
 #include <vector>
@@ -274,6 +274,8 @@ __global__ void __launch_bounds__(512, 1) k_noise_table(NoiseArgs a, int8_t *out
   for (uint32_t w = threadIdx.x; w < 65536; w += blockDim.x) out[w] = (int8_t)tab_sample(smem, w);
 }
 
+#include "products.cuh"
+
 // ---------------------------------------------------------------------------
 // Rows times S^T: out[r][l] = sum_j X[r][j] * St[l][j] for l < 8.
 // A warp owns a row; a lane takes 8-element chunks (16 bytes of X, one AES
@@ -298,206 +300,6 @@ LWE_DEV void warp_allreduce8(int acc[8]) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc[l] += __shfl_xor_sync(0xffffffffu, acc[l], o);
   }
-}
-
-// A S + E with A regenerated (KeyGen, Alg. 1, fused): persistent CTAs of
-// 16 warps fill the AES tables once and walk the rows (warp per row, lane
-// per 16-byte chunk = one AES block of A's counter layout).
-__global__ void __launch_bounds__(512, 1) k_mul_as_fused(MulAsArgs a) {
-  extern __shared__ uint32_t sT[];
-  pdl_trigger();
-  aes_fill_smem(sT, g_aes_img);
-  __syncthreads();
-  pdl_wait();
-  const AesTab tab = aes_tab(sT);
-  const uint32_t e = blockIdx.y;
-  uint32_t key[4], rk[44];
-  aes_load_key(a.seeds + (size_t)e * a.seed_stride, key);
-  aes_key_expand(tab, key, rk);
-  const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t n = a.n;
-  const uint32_t m = (1u << a.logq) - 1u, mm = m | (m << 16);
-  const int8_t *St = a.St + (size_t)e * a.st_stride;
-  const uint32_t rows = a.rows ? a.rows : n;
-  for (uint32_t i = blockIdx.x * 16 + warp; i < rows; i += gridDim.x * 16) {
-    int acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    // a lane's blocks step by 32 through the row: its 256-aligned counter
-    // window (the first two AES rounds, aes_ctr_run) changes every 8 blocks
-    AesCtrRun win;
-    uint64_t wcur = ~0ull;
-    for (uint32_t jc = lane; jc < n / 8; jc += 32) {
-      const uint64_t b = (uint64_t)(a.row0 + i) * (n / 8) + jc;
-      if ((b >> 8) != wcur) {
-        wcur = b >> 8;
-        win = aes_ctr_run(tab, rk, 0, b);
-      }
-      uint4 x = aes_ctr_run_block(tab, rk, win, (uint32_t)b & 255u);
-      x.x &= mm;
-      x.y &= mm;
-      x.z &= mm;
-      x.w &= mm;
-      dot8_chunk(x, St, n, 8 * jc, acc);
-    }
-    warp_allreduce8(acc);
-    if (lane == 0) {
-      uint32_t v[8];
-      const int8_t *E = a.E ? a.E + (size_t)e * a.e_stride + (size_t)i * 8 : nullptr;
-#pragma unroll
-      for (int l = 0; l < 8; l++) v[l] = (uint32_t)(acc[l] + (E ? (int)E[l] : 0)) & m;
-      const uint4 pk = make_uint4(v[0] | (v[1] << 16), v[2] | (v[3] << 16), v[4] | (v[5] << 16),
-                                  v[6] | (v[7] << 16));
-      *reinterpret_cast<uint4 *>(a.out + (size_t)e * a.out_stride + 16 * (size_t)i) = pk;
-      if (a.out2)
-        *reinterpret_cast<uint4 *>(a.out2 + (size_t)e * a.out2_stride + 16 * (size_t)i) = pk;
-    }
-  }
-}
-
-// A S + E with stored A (KeyGen, Alg. 1).  A warp computes AS_ROWS rows of
-// A together, so every 64-byte chunk of S^T it loads serves AS_ROWS rows,
-// and keeps two 16-byte chunks of each row in flight per lane (A streams
-// past L1; S^T stays there).  The 8 AS_ROWS partial sums of a lane are
-// reduced across the warp by recursive halving, which leaves lane L with
-// output L = (row L / 8, column L % 8) for one coalesced store.
-#define AS_ROWS 4
-
-LWE_DEV uint4 ld_stream_u4(const void *p) {
-  uint4 v;
-  asm("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
-      : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-      : "l"(p));
-  return v;
-}
-
-LWE_DEV void dot8_rows(const uint4 *x, const int8_t *__restrict__ St, uint32_t n, uint32_t j,
-                       int acc[AS_ROWS][8]) {
-#pragma unroll
-  for (int l = 0; l < 8; l++) {
-    const uint2 s = ld_nc_u2(St + (size_t)l * n + j);
-#pragma unroll
-    for (int r = 0; r < AS_ROWS; r++) {
-      acc[r][l] = __dp2a_lo((int)x[r].x, (int)s.x, acc[r][l]);
-      acc[r][l] = __dp2a_hi((int)x[r].y, (int)s.x, acc[r][l]);
-      acc[r][l] = __dp2a_lo((int)x[r].z, (int)s.y, acc[r][l]);
-      acc[r][l] = __dp2a_hi((int)x[r].w, (int)s.y, acc[r][l]);
-    }
-  }
-}
-
-// Row groups (tasks) are dealt out task = CTA + grid * (warp + 8 k), so
-// that with a grid of two CTAs per SM every SM streams the same share of A.
-__global__ void __launch_bounds__(256) k_mul_as_rows(MulAsArgs a) {
-  pdl_trigger();
-  pdl_wait();
-  const uint32_t e = blockIdx.y;
-  const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t n = a.n, nch = n / 8;
-  const uint32_t tasks = (a.rows ? a.rows : n) / AS_ROWS;  // rows: a multiple of AS_ROWS
-  const int8_t *St = a.St + (size_t)e * a.st_stride;
-  for (uint32_t task = blockIdx.x + gridDim.x * warp; task < tasks; task += gridDim.x * 8) {
-  const uint32_t i0 = task * AS_ROWS;
-  if (!LWE_BOUNDS(i0 + AS_ROWS <= (a.rows ? a.rows : n), 109)) continue;
-  const uint16_t *A0 = a.A + (size_t)e * a.a_stride + (size_t)i0 * n;
-  int acc[AS_ROWS][8];
-#pragma unroll
-  for (int r = 0; r < AS_ROWS; r++)
-#pragma unroll
-    for (int l = 0; l < 8; l++) acc[r][l] = 0;
-  for (uint32_t jc = lane; jc < nch; jc += 64) {
-    const bool two = jc + 32 < nch;
-    uint4 x0[AS_ROWS], x1[AS_ROWS];
-#pragma unroll
-    for (int r = 0; r < AS_ROWS; r++) x0[r] = ld_stream_u4(A0 + (size_t)r * n + 8 * (size_t)jc);
-#pragma unroll
-    for (int r = 0; r < AS_ROWS; r++)
-      x1[r] = two ? ld_stream_u4(A0 + (size_t)r * n + 8 * (size_t)(jc + 32)) : make_uint4(0, 0, 0, 0);
-    dot8_rows(x0, St, n, 8 * jc, acc);
-    if (two) dot8_rows(x1, St, n, 8 * (jc + 32), acc);
-  }
-  // recursive halving: at offset o a lane keeps the half of its values
-  // selected by lane bit o and adds the partner's copy of that half
-  int v[32];
-#pragma unroll
-  for (int r = 0; r < AS_ROWS; r++)
-#pragma unroll
-    for (int l = 0; l < 8; l++) v[8 * r + l] = acc[r][l];
-#pragma unroll
-  for (int o = 16; o >= 1; o >>= 1) {
-    const bool up = (lane & o) != 0;
-#pragma unroll
-    for (int j = 0; j < o; j++) {
-      const int send = up ? v[j] : v[j + o];
-      const int keep = up ? v[j + o] : v[j];
-      v[j] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-    }
-  }
-  const uint32_t r = lane >> 3, l = lane & 7, i = i0 + r;
-  const uint32_t m = (1u << a.logq) - 1u;
-  const int ev = a.E ? (int)a.E[(size_t)e * a.e_stride + (size_t)i * 8 + l] : 0;
-  const uint16_t val = (uint16_t)((uint32_t)(v[0] + ev) & m);
-  reinterpret_cast<uint16_t *>(a.out + (size_t)e * a.out_stride + 16 * (size_t)i)[l] = val;
-  if (a.out2) reinterpret_cast<uint16_t *>(a.out2 + (size_t)e * a.out2_stride + 16 * (size_t)i)[l] = val;
-  }
-}
-
-// The same for calls with few rows in all (one item, n up to a few
-// thousand): the kernel above then has less than one row group per warp and
-// each warp's chain of dependent loads sets the time.  Here a CTA takes one
-// row group and its 8 warps split the columns, so 8 times as many warps keep
-// loads in flight; their partial sums meet in shared memory.
-__global__ void __launch_bounds__(256) k_mul_as_split(MulAsArgs a) {
-  __shared__ int red[8][32];
-  pdl_trigger();
-  pdl_wait();
-  const uint32_t e = blockIdx.y, i0 = blockIdx.x * AS_ROWS;
-  const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t n = a.n, nch = n / 8;
-  const uint32_t c0 = warp * nch / 8, c1 = (warp + 1) * nch / 8;
-  const int8_t *St = a.St + (size_t)e * a.st_stride;
-  const uint16_t *A0 = a.A + (size_t)e * a.a_stride + (size_t)i0 * n;
-  int acc[AS_ROWS][8];
-#pragma unroll
-  for (int r = 0; r < AS_ROWS; r++)
-#pragma unroll
-    for (int l = 0; l < 8; l++) acc[r][l] = 0;
-  for (uint32_t jc = c0 + lane; jc < c1; jc += 64) {
-    const bool two = jc + 32 < c1;
-    uint4 x0[AS_ROWS], x1[AS_ROWS];
-#pragma unroll
-    for (int r = 0; r < AS_ROWS; r++) x0[r] = ld_stream_u4(A0 + (size_t)r * n + 8 * (size_t)jc);
-#pragma unroll
-    for (int r = 0; r < AS_ROWS; r++)
-      x1[r] = two ? ld_stream_u4(A0 + (size_t)r * n + 8 * (size_t)(jc + 32)) : make_uint4(0, 0, 0, 0);
-    dot8_rows(x0, St, n, 8 * jc, acc);
-    if (two) dot8_rows(x1, St, n, 8 * (jc + 32), acc);
-  }
-  int v[32];
-#pragma unroll
-  for (int r = 0; r < AS_ROWS; r++)
-#pragma unroll
-    for (int l = 0; l < 8; l++) v[8 * r + l] = acc[r][l];
-#pragma unroll
-  for (int o = 16; o >= 1; o >>= 1) {
-    const bool up = (lane & o) != 0;
-#pragma unroll
-    for (int j = 0; j < o; j++) {
-      const int send = up ? v[j] : v[j + o];
-      const int keep = up ? v[j + o] : v[j];
-      v[j] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-    }
-  }
-  red[warp][lane] = v[0];
-  __syncthreads();
-  if (warp != 0) return;
-  int sum = 0;
-#pragma unroll
-  for (int w = 0; w < 8; w++) sum += red[w][lane];
-  const uint32_t r = lane >> 3, l = lane & 7, i = i0 + r;
-  const uint32_t m = (1u << a.logq) - 1u;
-  const int ev = a.E ? (int)a.E[(size_t)e * a.e_stride + (size_t)i * 8 + l] : 0;
-  const uint16_t val = (uint16_t)((uint32_t)(sum + ev) & m);
-  reinterpret_cast<uint16_t *>(a.out + (size_t)e * a.out_stride + 16 * (size_t)i)[l] = val;
-  if (a.out2) reinterpret_cast<uint16_t *>(a.out2 + (size_t)e * a.out2_stride + 16 * (size_t)i)[l] = val;
 }
 
 // Decrypt (Alg. 3): warp r of CTA e computes row r of M = C - B' S and the
@@ -541,303 +343,6 @@ __global__ void __launch_bounds__(256) k_decrypt(DecryptArgs a) {
     }
     uint8_t *mu = a.mu + (size_t)e * 32 + r * Bb;
     for (uint32_t t = 0; t < Bb; t++) mu[t] = (uint8_t)(bits >> (8 * t));
-  }
-}
-
-// S' A (+ E') for one or more items on the CUDA cores (Alg. 2), A stored
-// (LDG.128 of 8 columns per row) or regenerated (one AES block per row and
-// 8 columns, the counter layout of A).  CTA = (256-column block, row
-// split, item): lane l owns columns 8 l .. 8 l + 7 of the block, warp w the
-// row pairs (2p, 2p + 1) with p = w (mod 8); the pair's S' bytes are staged
-// in shared memory so that one dp2a multiplies two rows.  The warps' sums
-// meet in shared memory; when a call has few items the rows are split over
-// a cluster of R CTAs whose partial sums are added through distributed
-// shared memory, so no global workspace is needed.  Then E' is added and
-// the row stored, or (CMP) compared with the received ciphertext.
-#define SA_PAIRS 512  // row pairs of S' staged at a time (8 KB)
-
-LWE_DEV uint32_t cluster_map(const void *p, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
-               : "=r"(r)
-               : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
-  return r;
-}
-LWE_DEV int ld_cluster_s32(uint32_t addr) {
-  int v;
-  asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
-  return v;
-}
-LWE_DEV void cluster_barrier() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::
-                   : "memory");
-}
-
-// word q of pair p: S'[2q][2p], S'[2q][2p+1], S'[2q+1][2p], S'[2q+1][2p+1]
-LWE_DEV void sa_stage(const int8_t *S, uint32_t n, uint32_t c0, uint32_t cn, uint4 *sP,
-                      uint32_t tid, uint32_t nt) {
-  for (uint32_t q = tid; q < cn; q += nt) {
-    const uint32_t i = 2 * (c0 + q);
-    uint32_t w[4];
-#pragma unroll
-    for (int kk = 0; kk < 4; kk++) {
-      const uint32_t lo = *reinterpret_cast<const uint16_t *>(S + (size_t)(2 * kk) * n + i);
-      const uint32_t hi = *reinterpret_cast<const uint16_t *>(S + (size_t)(2 * kk + 1) * n + i);
-      w[kk] = lo | (hi << 16);
-    }
-    sP[q] = make_uint4(w[0], w[1], w[2], w[3]);
-  }
-}
-
-// One column c of both rows of a pair as two 16-bit halves, times the pair's
-// S' bytes for all 8 rows k: acc[k] += S'[k][2p] A[2p][c] + S'[k][2p+1] A[2p+1][c]
-LWE_DEV void sa_mac_col(int pk, const uint4 sp, int *acc_c /* [8] stride */, int stride) {
-  const uint32_t sw[4] = {sp.x, sp.y, sp.z, sp.w};
-#pragma unroll
-  for (int q = 0; q < 4; q++) {
-    acc_c[(2 * q) * stride] = __dp2a_lo(pk, (int)sw[q], acc_c[(2 * q) * stride]);
-    acc_c[(2 * q + 1) * stride] = __dp2a_hi(pk, (int)sw[q], acc_c[(2 * q + 1) * stride]);
-  }
-}
-
-// The CTA's (and with R > 1 the cluster's) sums red[k][c][32] (column
-// 8 lane + c of the block) are finished: + E', mod q, store or compare.
-template <bool CMP>
-LWE_DEV void sa_epilogue(const MulSaArgs &a, int *red, uint32_t cb, uint32_t rsplit, uint32_t R,
-                         uint32_t e, uint32_t tid, uint32_t nt) {
-  const uint32_t n = a.n, mq = (1u << a.logq) - 1u;
-  const uint32_t share = 2048 / R;
-  uint32_t diff = 0;
-  for (uint32_t v = rsplit * share + tid; v < (rsplit + 1) * share; v += nt) {
-    const uint32_t k = v >> 8, col = v & 255;
-    const uint32_t idx = k * 256 + (col & 7) * 32 + (col >> 3);
-    int sum = 0;
-    if (R > 1) {
-      for (uint32_t r = 0; r < R; r++) sum += ld_cluster_s32(cluster_map(red + idx, r));
-    } else {
-      sum = red[idx];
-    }
-    const uint32_t j = cb * 256 + col;
-    if (j < n) {
-      if (a.E) sum += a.E[(size_t)e * a.e_stride + (size_t)k * n + j];
-      const uint32_t val = (uint32_t)sum & mq;
-      uint16_t *o = reinterpret_cast<uint16_t *>(a.out + (size_t)e * a.out_stride) + (size_t)k * n + j;
-      if (CMP)
-        diff |= val ^ (uint32_t)*o;
-      else
-        *o = (uint16_t)val;
-    }
-  }
-  if (CMP) {
-    diff = __reduce_or_sync(0xffffffffu, diff);
-    if ((tid & 31) == 0 && diff) atomicOr(a.flags + e, 1u);
-  }
-}
-
-template <bool CMP>
-__global__ void __launch_bounds__(256) k_sa(MulSaArgs a) {
-  extern __shared__ uint4 sm4[];
-  pdl_trigger();
-  pdl_wait();
-  uint4 *sP = sm4;
-  int *red = reinterpret_cast<int *>(sm4 + SA_PAIRS);
-  const uint32_t cb = blockIdx.x, rsplit = blockIdx.y, R = gridDim.y, e = blockIdx.z;
-  const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const uint32_t n = a.n;
-  const uint32_t j0 = cb * 256 + 8 * lane;
-  const bool jv = j0 < n;  // n and j0 are multiples of 8: a chunk is all in or all out
-  for (uint32_t i = tid; i < 2048; i += 256) red[i] = 0;
-  const int8_t *S = a.S + (size_t)e * a.s_stride;
-  const uint32_t p0 = a.row0 / 2, p1 = (a.row1 ? a.row1 : n) / 2;
-  // a stored row block starts at row row0
-  const uint16_t *Aitem = a.A_ptrs ? a.A_ptrs[e] : a.A;
-  const uint32_t r0 = a.row0;
-  const uint32_t per = (p1 - p0 + R - 1) / R;
-  const uint32_t pb = min(p1, p0 + rsplit * per), pe = min(p1, pb + per);
-  int acc[8][8];
-#pragma unroll
-  for (int k = 0; k < 8; k++)
-#pragma unroll
-    for (int c = 0; c < 8; c++) acc[k][c] = 0;
-  auto row_chunk = [&](uint32_t i) -> uint4 {
-    return jv && LWE_BOUNDS(i >= r0 && i < (a.row1 ? a.row1 : n), 110)
-               ? ld_nc_u4(Aitem + (size_t)(i - r0) * n + j0)
-               : make_uint4(0, 0, 0, 0);
-  };
-  auto mac_pair = [&](const uint4 x0, const uint4 x1, const uint4 sp) {
-    const uint32_t w0[4] = {x0.x, x0.y, x0.z, x0.w}, w1[4] = {x1.x, x1.y, x1.z, x1.w};
-#pragma unroll
-    for (int c = 0; c < 8; c++) {
-      // column c of both rows as two 16-bit halves (signed: same residues)
-      const int pk = (int)__byte_perm(w0[c >> 1], w1[c >> 1], (c & 1) ? 0x7632 : 0x5410);
-      sa_mac_col(pk, sp, &acc[0][c], 8);
-    }
-  };
-  for (uint32_t c0 = pb; c0 < pe; c0 += SA_PAIRS) {
-    const uint32_t cn = min((uint32_t)SA_PAIRS, pe - c0);
-    __syncthreads();
-    sa_stage(S, n, c0, cn, sP, tid, 256);
-    __syncthreads();
-    uint32_t q = warp;
-    for (; q + 24 < cn; q += 32) {  // four pairs (eight rows) in flight
-      const uint32_t i = 2 * (c0 + q);
-      uint4 x[8];
-#pragma unroll
-      for (int u = 0; u < 4; u++) {
-        x[2 * u] = row_chunk(i + 16 * u);
-        x[2 * u + 1] = row_chunk(i + 16 * u + 1);
-      }
-#pragma unroll
-      for (int u = 0; u < 4; u++) mac_pair(x[2 * u], x[2 * u + 1], sP[q + 8 * u]);
-    }
-    for (; q + 8 < cn; q += 16) {  // two pairs in flight
-      const uint32_t i = 2 * (c0 + q), i2 = i + 16;
-      const uint4 x0 = row_chunk(i), x1 = row_chunk(i + 1);
-      const uint4 y0 = row_chunk(i2), y1 = row_chunk(i2 + 1);
-      mac_pair(x0, x1, sP[q]);
-      mac_pair(y0, y1, sP[q + 8]);
-    }
-    if (q < cn) {
-      const uint32_t i = 2 * (c0 + q);
-      mac_pair(row_chunk(i), row_chunk(i + 1), sP[q]);
-    }
-  }
-  // the CTA's sum: red[k][c][lane] (column 8 lane + c)
-#pragma unroll
-  for (int k = 0; k < 8; k++)
-#pragma unroll
-    for (int c = 0; c < 8; c++) atomicAdd(&red[k * 256 + c * 32 + lane], acc[k][c]);
-  __syncthreads();
-  if (R > 1) cluster_barrier();  // every CTA of the cluster has its partial sum
-  sa_epilogue<CMP>(a, red, cb, rsplit, R, e, tid, 256);
-  if (R > 1) cluster_barrier();  // no CTA leaves while others read its shared memory
-}
-
-// The same product with A regenerated (the AES tables in shared memory): 16
-// warps; a lane pair shares one 8-column chunk, lane s of the pair
-// encrypting row 2p + s of each row pair and the two swapping half blocks,
-// so each lane holds 4 columns of both rows (32 sums, room for 16 warps).
-// Warps 0-7 take columns 0-127 of the CTA's block, warps 8-15 columns
-// 128-255.
-template <bool CMP>
-__global__ void __launch_bounds__(512, 1) k_sa_fused(MulSaArgs a) {
-  extern __shared__ uint4 sm4[];
-  uint8_t *base = reinterpret_cast<uint8_t *>(sm4);
-  uint4 *sP = reinterpret_cast<uint4 *>(base + AES_SMEM_BYTES);
-  int *red = reinterpret_cast<int *>(base + AES_SMEM_BYTES + SA_PAIRS * 16);
-  const uint32_t cb = blockIdx.x, rsplit = blockIdx.y, R = gridDim.y, e = blockIdx.z;
-  const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const uint32_t rw = warp & 7, half = warp >> 3, s = lane & 1;
-  const uint32_t n = a.n;
-  const uint32_t chunk = cb * 32 + half * 16 + (lane >> 1);  // 8-column chunk index
-  const uint32_t j0 = 8 * chunk;
-  const bool jv = j0 < n;
-  pdl_trigger();
-  for (uint32_t i = tid; i < 2048; i += 512) red[i] = 0;
-  uint32_t *sT = reinterpret_cast<uint32_t *>(base);
-  aes_fill_smem(sT, g_aes_img);
-  __syncthreads();
-  pdl_wait();
-  const AesTab tab = aes_tab(sT);
-  uint32_t key[4], rk[44];
-  aes_load_key(a.seed_ptrs ? a.seed_ptrs[e] + a.seed_off : a.seedA, key);
-  aes_key_expand(tab, key, rk);
-  const uint32_t mq = (1u << a.logq) - 1u, mm = mq | (mq << 16);
-  const int8_t *S = a.S + (size_t)e * a.s_stride;
-  const uint32_t p0 = a.row0 / 2, p1 = (a.row1 ? a.row1 : n) / 2;
-  const uint32_t per = (p1 - p0 + R - 1) / R;
-  const uint32_t pb = min(p1, p0 + rsplit * per), pe = min(p1, pb + per);
-  int acc[8][4];
-#pragma unroll
-  for (int k = 0; k < 8; k++)
-#pragma unroll
-    for (int c = 0; c < 4; c++) acc[k][c] = 0;
-  for (uint32_t c0 = pb; c0 < pe; c0 += SA_PAIRS) {
-    const uint32_t cn = min((uint32_t)SA_PAIRS, pe - c0);
-    __syncthreads();
-    sa_stage(S, n, c0, cn, sP, tid, 512);
-    __syncthreads();
-    for (uint32_t q = rw; q < cn; q += 8) {
-      const uint32_t i = 2 * (c0 + q) + s;  // this lane's row of the pair
-      uint4 x = make_uint4(0, 0, 0, 0);
-      if (jv) {
-        x = aes_ctr_block(tab, rk, 0, (uint64_t)i * (n / 8) + chunk);
-        x.x &= mm;
-        x.y &= mm;
-        x.z &= mm;
-        x.w &= mm;
-      }
-      // lane 0 of the pair keeps columns 0-3 of its row and takes columns
-      // 0-3 of row 2p+1; lane 1 keeps columns 4-7 of row 2p+1 and takes 4-7
-      // of row 2p
-      const uint32_t g0 = s ? x.x : x.z, g1 = s ? x.y : x.w;
-      const uint32_t r0 = __shfl_xor_sync(0xffffffffu, g0, 1);
-      const uint32_t r1 = __shfl_xor_sync(0xffffffffu, g1, 1);
-      const uint32_t a0 = s ? r0 : x.x, a1 = s ? r1 : x.y;  // row 2p, my 4 columns
-      const uint32_t b0 = s ? x.z : r0, b1 = s ? x.w : r1;  // row 2p+1
-      const uint4 sp = sP[q];
-      sa_mac_col((int)__byte_perm(a0, b0, 0x5410), sp, &acc[0][0], 4);
-      sa_mac_col((int)__byte_perm(a0, b0, 0x7632), sp, &acc[0][1], 4);
-      sa_mac_col((int)__byte_perm(a1, b1, 0x5410), sp, &acc[0][2], 4);
-      sa_mac_col((int)__byte_perm(a1, b1, 0x7632), sp, &acc[0][3], 4);
-    }
-  }
-  // column of the block owned by (half, lane): 128 half + 8 (lane / 2) + 4 s + c
-  const uint32_t cl = half * 16 + (lane >> 1);  // chunk within the block (0..31)
-#pragma unroll
-  for (int k = 0; k < 8; k++)
-#pragma unroll
-    for (int c = 0; c < 4; c++) atomicAdd(&red[k * 256 + (4 * s + c) * 32 + cl], acc[k][c]);
-  __syncthreads();
-  if (R > 1) cluster_barrier();
-  sa_epilogue<CMP>(a, red, cb, rsplit, R, e, tid, 512);
-  if (R > 1) cluster_barrier();
-}
-
-// ---------------------------------------------------------------------------
-// V = S' B + E'' and C = V + Enc(mu) (Alg. 2); CTA per item, warp per row k.
-// ---------------------------------------------------------------------------
-template <bool CMP>
-__global__ void __launch_bounds__(256) k_v_encode(VEncArgs a) {
-  pdl_trigger();
-  pdl_wait();
-  const uint32_t e = blockIdx.x;
-  const uint32_t k = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t n = a.n;
-  const int8_t *S = a.S + (size_t)e * a.s_stride + (size_t)k * n;
-  const uint8_t *pk = a.pk_ptrs ? a.pk_ptrs[e] + a.pk_off : a.pk;
-  const uint16_t *Bm = reinterpret_cast<const uint16_t *>(pk + 16);
-  int acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  for (uint32_t i = lane; i < n; i += 32) {
-    const int s = S[i];
-    const uint4 b = ld_nc_u4(Bm + 8 * (size_t)i);
-    const uint32_t w[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-    for (int l = 0; l < 8; l++) acc[l] += s * (int)((w[l >> 1] >> (16 * (l & 1))) & 0xffffu);
-  }
-  warp_allreduce8(acc);
-  if (lane == 0) {
-    const uint32_t D = a.logq, Bb = a.B, m = (1u << D) - 1u;
-    const int8_t *Epp = a.Epp + (size_t)e * a.epp_stride + 8 * k;
-    const uint8_t *mu = a.mu + (size_t)e * 32 + k * Bb;
-    uint32_t bits = 0;
-    for (uint32_t t = 0; t < Bb; t++) bits |= (uint32_t)mu[t] << (8 * t);
-    uint32_t c[8];
-#pragma unroll
-    for (int l = 0; l < 8; l++) {
-      const uint32_t sym = (bits >> (l * Bb)) & ((1u << Bb) - 1u);
-      c[l] = ((uint32_t)(acc[l] + Epp[l]) + (sym << (D - Bb))) & m;
-    }
-    const uint4 pk = make_uint4(c[0] | (c[1] << 16), c[2] | (c[3] << 16), c[4] | (c[5] << 16),
-                                c[6] | (c[7] << 16));
-    uint4 *dst = reinterpret_cast<uint4 *>(a.ct + (size_t)e * a.ct_bytes + 16 * (size_t)n + 16 * k);
-    if (CMP) {
-      const uint4 old = *dst;
-      const uint32_t diff = (old.x ^ pk.x) | (old.y ^ pk.y) | (old.z ^ pk.z) | (old.w ^ pk.w);
-      if (diff) atomicOr(a.flags + e, 1u);
-    } else {
-      *dst = pk;
-    }
   }
 }
 
@@ -1725,6 +1230,60 @@ cudaError_t lwe_upload_aes_table(const uint32_t T0[256]) {
   return cudaMemcpyToSymbol(g_aes_img, img.data(), AES_TABLE_WORDS * sizeof(uint32_t));
 }
 
+// CTAs of the AES product kernels (one per SM) that run at once in clusters
+// of R, per device: clusters do not straddle GPCs, so on a 152-SM GB300 not
+// every R uses every SM.  Filled by lwe_kernel_smem_setup.
+static uint32_t g_cluster_slots[128][9];
+
+static uint32_t cluster_slots(uint32_t R, uint32_t sms) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 128) return sms / R * R;
+  const uint32_t n = g_cluster_slots[dev][R];
+  return n ? n : sms / R * R;
+}
+
+static cudaError_t query_cluster_slots() {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess || dev < 0 || dev >= 128) return e;
+  for (uint32_t R = 1; R <= 8; R++) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(1, R, 1);
+    cfg.blockDim = dim3(512, 1, 1);
+    cfg.dynamicSmemBytes = PRD_SMEM;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 1;
+    at[0].val.clusterDim.y = R;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    e = cudaOccupancyMaxActiveClusters(&n, k_sa_gen<false>, &cfg);
+    if (e != cudaSuccess) return e;
+    g_cluster_slots[dev][R] = (uint32_t)n * R;
+  }
+  return cudaSuccess;
+}
+
+// How many ways (1 .. 8, one cluster) to split each of `tiles` equal pieces
+// of `work` units so that the last wave wastes least; every CTA has a fixed
+// cost of `fixed` units.
+static uint32_t best_split(uint64_t tiles, uint32_t work, uint32_t fixed, uint32_t sms) {
+  uint32_t best = 1;
+  uint64_t best_cost = ~0ull;
+  for (uint32_t R = 1; R <= 8 && R <= work; R++) {
+    const uint32_t slots = std::max(R, cluster_slots(R, sms));
+    const uint64_t waves = (tiles * R + slots - 1) / slots;
+    const uint64_t cost = waves * ((work + R - 1) / R + fixed);
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = R;
+    }
+  }
+  return best;
+}
+
 cudaError_t lwe_kernel_smem_setup() {
   cudaError_t e;
   e = cudaFuncSetAttribute(k_expand_A, cudaFuncAttributeMaxDynamicSharedMemorySize, AES_SMEM_BYTES);
@@ -1734,12 +1293,15 @@ cudaError_t lwe_kernel_smem_setup() {
   e = cudaFuncSetAttribute(k_noise_table, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            NOISE_SMEM_BYTES);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_mul_as_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, AES_SMEM_BYTES);
+  e = cudaFuncSetAttribute(k_mul_as_gen, cudaFuncAttributeMaxDynamicSharedMemorySize, AS_GEN_SMEM);
   if (e != cudaSuccess) return e;
-  const int fused_smem = AES_SMEM_BYTES + SA_PAIRS * 16 + 2048 * 4;
-  e = cudaFuncSetAttribute(k_sa_fused<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, fused_smem);
+  e = cudaFuncSetAttribute(k_mul_as_gen_split, cudaFuncAttributeMaxDynamicSharedMemorySize, PRD_SMEM);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_sa_fused<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, fused_smem);
+  e = cudaFuncSetAttribute(k_sa_gen<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PRD_SMEM);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(k_sa_gen<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, PRD_SMEM);
+  if (e != cudaSuccess) return e;
+  e = query_cluster_slots();
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_probe_aes, cudaFuncAttributeMaxDynamicSharedMemorySize, AES_SMEM_BYTES);
   if (e != cudaSuccess) return e;
@@ -1771,21 +1333,39 @@ void launch_noise(const NoiseArgs &a, int num_sms, cudaStream_t st) {
 }
 
 void launch_mul_as(const MulAsArgs &a, uint32_t count, bool fused, int num_sms, cudaStream_t st) {
-  const uint32_t rows = a.rows ? a.rows : a.n;
-  if (fused) {
-    const uint32_t per_item = std::max<uint32_t>(1u, (uint32_t)std::max(num_sms, 1) / count);
-    dim3 grid(std::min((rows + 15) / 16, per_item), count);
-    launch_k(k_mul_as_fused, grid, 512, AES_SMEM_BYTES, st, a);
-  } else if ((uint64_t)count * (rows / AS_ROWS) < 4ull * 16 * (uint64_t)std::max(num_sms, 1)) {
-    // fewer than ~4 row groups per warp of the grid below: split columns
-    launch_k(k_mul_as_split, dim3(rows / AS_ROWS, count), 256, 0, st, a);
-  } else {
-    // two CTAs per SM in all, spread over the items
-    const uint32_t want = (rows / AS_ROWS + 7) / 8;
-    const uint32_t share = std::max<uint32_t>(1u, 2u * (uint32_t)std::max(num_sms, 1) / count);
-    dim3 grid(std::min(want, share), count);
-    launch_k(k_mul_as_rows, grid, 256, 0, st, a);
+  const uint32_t rows = a.rows ? a.rows : a.n, sms = (uint32_t)std::max(num_sms, 1);
+  if (!fused) {
+    // 8 warps per 16-row tile, but 4 where 8 (three CTAs per SM) would leave a
+    // short second wave that 4 (six per SM) take along: n = 8192, 512 tiles,
+    // 28.4 us with 8 and 25.7 with 4; n = 16384, 1024 tiles, 95.5 and 101.8
+    const uint64_t tiles = (uint64_t)(rows / 16) * count;
+    if (tiles > 3ull * sms && tiles <= 6ull * sms)
+      launch_k(k_mul_as<4>, dim3(rows / 16, count), 128, 0, st, a);
+    else
+      launch_k(k_mul_as<8>, dim3(rows / 16, count), 256, 0, st, a);
+    return;
   }
+  const uint64_t units = (uint64_t)count * (rows / 16);
+  if (units >= 32ull * sms) {
+    launch_k(k_mul_as_gen, sms, 512, AS_GEN_SMEM, st, a, count);
+    return;
+  }
+  // clusters of R CTAs walk the 16-row tiles of each item
+  const uint32_t tiles = rows / 16, groups = (a.n / 8 + 3) / 4;  // groups of 4 chunks per tile
+  uint32_t best_R = 1, best_G = 1;
+  uint64_t best_cost = ~0ull;
+  for (uint32_t R = 1; R <= 8; R++) {
+    const uint32_t slots = std::max(R, cluster_slots(R, sms));
+    const uint32_t G = std::min(tiles, std::max<uint32_t>(1u, slots / (R * count)));
+    const uint64_t ctas = (uint64_t)R * G * count;
+    const uint64_t cost = ((ctas + slots - 1) / slots) * ((tiles + G - 1) / G) * ((groups + R - 1) / R + 3);
+    if (cost < best_cost) {
+      best_cost = cost;
+      best_R = R;
+      best_G = G;
+    }
+  }
+  launch_k_cluster(k_mul_as_gen_split, dim3(best_R, best_G, count), 512, PRD_SMEM, st, best_R, a);
 }
 
 void launch_decrypt(const DecryptArgs &a, uint32_t count, cudaStream_t st) {
@@ -1794,16 +1374,36 @@ void launch_decrypt(const DecryptArgs &a, uint32_t count, cudaStream_t st) {
 
 void launch_mul_sa(const MulSaArgs &a, uint32_t items, bool fused, bool cmp, int num_sms,
                    cudaStream_t st) {
-  // rows split over a cluster of R CTAs (R a power of two <= 8) until the
-  // grid holds about two CTAs per SM (one with the AES tables)
-  const uint32_t cbs = (a.n + 255) / 256;
-  const uint32_t target = (fused ? 1u : 2u) * (uint32_t)std::max(num_sms, 1);
-  const uint32_t pairs = ((a.row1 ? a.row1 : a.n) - a.row0) / 2;
-  uint32_t R = 1;
-  while (R < 8 && (uint64_t)cbs * items * R < target && pairs / (2 * R) >= 64) R <<= 1;
+  const uint32_t sms = (uint32_t)std::max(num_sms, 1);
+  const uint32_t steps = ((a.row1 ? a.row1 : a.n) - a.row0) / 16;  // 16-row steps
+  uint32_t R, cgs = 1, cbs = (a.n + 63) / 64;
+  if (fused) {
+    R = best_split((uint64_t)cbs * items, steps, 14, sms);
+  } else {
+    // column groups per CTA and row split: few waves of two CTAs per SM (90
+    // registers), counting 64 steps for a CTA's start and end, and two row
+    // steps per warp at least; of equals the narrowest, whose clusters are
+    // small.  A from memory, n = 8192: 256 CTAs as 1 x 2, 2 x 4 or 4 x 8 take
+    // 31.3, 32.6 and 33.2 us, 384 as 1 x 3 43.6; n = 12000: 282 as 2 x 3 59.9,
+    // 4 x 6 106 (clusters of 6 do not fill the GPCs); 16384: 1 x 1 100.7
+    const uint32_t slots = 2 * sms;
+    uint64_t best_cost = ~0ull;
+    R = 1;
+    for (uint32_t g = 1; g <= 4; g *= 2)
+      for (uint32_t r = 1; r <= 8 && (r == 1 || steps * g >= 16 * r); r++) {
+        const uint64_t ctas = (uint64_t)((a.n + 64 * g - 1) / (64 * g)) * items * r;
+        const uint64_t cost = (ctas + slots - 1) / slots * ((uint64_t)steps * g / r + 64);
+        if (cost < best_cost) {
+          best_cost = cost;
+          cgs = g;
+          R = r;
+        }
+      }
+    cbs = (a.n + 64 * cgs - 1) / (64 * cgs);
+  }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(cbs, R, items);
-  cfg.dynamicSmemBytes = (fused ? AES_SMEM_BYTES : 0) + SA_PAIRS * 16 + 2048 * 4;
+  cfg.gridDim = dim3(cbs + (a.vcols ? 1 : 0), R, items);
+  cfg.dynamicSmemBytes = fused ? PRD_SMEM : 0;
   cfg.blockDim = dim3(fused ? 512 : 256, 1, 1);
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
@@ -1817,22 +1417,15 @@ void launch_mul_sa(const MulSaArgs &a, uint32_t items, bool fused, bool cmp, int
   cfg.numAttrs = R > 1 ? 2 : 1;
   if (fused) {
     if (cmp)
-      cudaLaunchKernelEx(&cfg, k_sa_fused<true>, a);
+      cudaLaunchKernelEx(&cfg, k_sa_gen<true>, a);
     else
-      cudaLaunchKernelEx(&cfg, k_sa_fused<false>, a);
+      cudaLaunchKernelEx(&cfg, k_sa_gen<false>, a);
   } else {
     if (cmp)
-      cudaLaunchKernelEx(&cfg, k_sa<true>, a);
+      cudaLaunchKernelEx(&cfg, k_sa<true>, a, cgs);
     else
-      cudaLaunchKernelEx(&cfg, k_sa<false>, a);
+      cudaLaunchKernelEx(&cfg, k_sa<false>, a, cgs);
   }
-}
-
-void launch_v_encode(const VEncArgs &a, uint32_t count, bool cmp, cudaStream_t st) {
-  if (cmp)
-    launch_k(k_v_encode<true>, count, 256, 0, st, a);
-  else
-    launch_k(k_v_encode<false>, count, 256, 0, st, a);
 }
 
 void launch_keygen_seeds(const KeygenSeedArgs &a, uint32_t warp_max, cudaStream_t st) {

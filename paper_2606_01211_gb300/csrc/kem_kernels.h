@@ -80,26 +80,17 @@ struct MulSaArgs {
   uint64_t out_stride;
   uint32_t *flags;       // compare mode: atomicOr(flags[e], 1) on mismatch
   const uint16_t *const *A_ptrs;  // per-item stored A (then A unused)
-  const uint8_t *const *seed_ptrs;  // per-item seedA at seed_ptrs[e] + seed_off (fused)
-  uint64_t seed_off;
+  const uint8_t *const *key_ptrs;  // per-item public key at key_ptrs[e] + key_off
+  uint64_t key_off;                // (its seedA when A is regenerated, its B for vcols)
   // row block: the sum runs over rows [row0, row1) of A only (row1 = 0: n);
   // a stored A then points at row row0 (rows of length n)
   uint32_t row0, row1;
-};
-
-struct VEncArgs {
-  const uint8_t *pk;     // seedA || B (n x 8 uint16)
-  const uint8_t *const *pk_ptrs;  // per-item public key at pk_ptrs[e] + pk_off
-  uint64_t pk_off;
-  const int8_t *S;       // item e: S' (8 x n) at S + e * s_stride
-  uint64_t s_stride;
+  // vcols: C = S' B + E'' + Enc(mu) too, at out + e*out_stride + 16 n
+  const uint8_t *pk;     // seedA || B (n x 8 uint16), without key_ptrs
   const int8_t *Epp;     // item e: E'' (8 x 8) at Epp + e * epp_stride
   uint64_t epp_stride;
   const uint8_t *mu;     // 32-byte slot per item
-  uint8_t *ct;           // item e at ct + e * ct_bytes; C at +16n
-  uint64_t ct_bytes;
-  uint32_t *flags;
-  uint32_t n, logq, B, pad;
+  uint32_t B, vcols;
 };
 
 struct KeygenSeedArgs {
@@ -177,7 +168,6 @@ void launch_mul_as(const MulAsArgs &a, uint32_t count, bool fused, int num_sms, 
 void launch_decrypt(const DecryptArgs &a, uint32_t count, cudaStream_t st);
 void launch_mul_sa(const MulSaArgs &a, uint32_t items, bool fused, bool cmp, int num_sms,
                    cudaStream_t st);
-void launch_v_encode(const VEncArgs &a, uint32_t count, bool cmp, cudaStream_t st);
 // launches of at most warp_max items hash with one Keccak state per warp
 void launch_keygen_seeds(const KeygenSeedArgs &a, uint32_t warp_max, cudaStream_t st);
 void launch_derive(const DeriveArgs &a, uint32_t warp_max, cudaStream_t st);

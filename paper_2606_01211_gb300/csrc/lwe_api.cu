@@ -144,7 +144,7 @@ uint32_t mu_bytes(const lwe_params &p) { return 8 * p.B; }
 
 const char *kKernelNames[KID_COUNT] = {
     "k_expand_A", "k_noise",    "k_keygen_seeds", "k_mul_as", "k_decrypt",
-    "k_sa",       "k_sa_fused", "k_v_encode",     "k_tree",   "k_final_key",
+    "k_sa",       "k_sa_fused", "k_tree",         "k_final_key",
     "k_derive",   "k_limbs",    "k_gemm_tc",      "k_tree_warp"};
 
 }  // namespace
@@ -446,34 +446,20 @@ int run_encrypt(lwe_ctx *c, const uint8_t *pk, const uint16_t *A, uint32_t count
   sa.out = ct;
   sa.out_stride = ct_bytes(c->p);
   sa.flags = c->flags;
+  sa.pk = pk;
+  sa.Epp = c->epp;
+  sa.epp_stride = 64;
+  sa.mu = c->mu;
+  sa.B = c->p.B;
+  sa.vcols = 1;
   bool fused = A == nullptr;
   if (ik) {
     sa.A_ptrs = ik->A_ptrs;
-    sa.seed_ptrs = ik->ptrs;
-    sa.seed_off = ik->pk_off;
+    sa.key_ptrs = ik->ptrs;
+    sa.key_off = ik->pk_off;
     fused = ik->A_ptrs == nullptr;
   }
   LAUNCH(c, fused ? KID_MUL_SA_FUSED : KID_MUL_SA, st, launch_mul_sa(sa, count, fused, cmp, c->num_sms, st));
-
-  VEncArgs va;
-  memset(&va, 0, sizeof va);
-  va.pk = pk;
-  if (ik) {
-    va.pk_ptrs = ik->ptrs;
-    va.pk_off = ik->pk_off;
-  }
-  va.S = c->sp8;
-  va.s_stride = 8ull * n;
-  va.Epp = c->epp;
-  va.epp_stride = 64;
-  va.mu = c->mu;
-  va.ct = ct;
-  va.ct_bytes = ct_bytes(c->p);
-  va.flags = c->flags;
-  va.n = n;
-  va.logq = c->p.logq;
-  va.B = c->p.B;
-  LAUNCH(c, KID_V_ENCODE, st, launch_v_encode(va, count, cmp, st));
   return check_launch();
 }
 

@@ -1,0 +1,57 @@
+"""The products of one request (csrc/products.cuh) against the oracle, bit for
+bit, at the sizes where their tiles can go wrong: n below one tile, row counts
+that are odd multiples of 16 (the second half of a 32-row tile absent, an odd
+number of 16-row steps), column counts that are no multiple of a 32-column
+chunk group or a 64-column group, S of the full int8 range, and the schedule
+for many regenerated items."""
+import numpy as np
+import pytest
+import torch
+
+from gpu_util import O, as_u16, dev, host, lwe, master_seeds, params
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _device():
+    assert torch.cuda.is_available()
+    torch.cuda.set_device(0)
+
+
+@pytest.mark.parametrize("n", [16, 48, 80, 640, 976, 1008, 2064, 4112])
+@pytest.mark.parametrize("stored", [True, False])
+@pytest.mark.parametrize("logq,k,amp", [(16, 8, 12), (15, 24, 127)])
+def test_products_match_oracle(n, stored, logq, k, amp):
+    r = np.random.default_rng(n + k)
+    seed = r.integers(0, 256, 16, dtype=np.uint8)
+    A_o = O.expand_A(bytes(seed), n, logq)
+    St = r.integers(-amp - 1, amp + 1, size=(8, n)).astype(np.int8)
+    E = r.integers(-amp - 1, amp + 1, size=(n, 8)).astype(np.int8)
+    S = r.integers(-amp - 1, amp + 1, size=(k, n)).astype(np.int8)
+    E2 = r.integers(-amp - 1, amp + 1, size=(k, n)).astype(np.int8)
+    A = dev(A_o.view(np.int16)) if stored else None
+    sd = None if stored else dev(seed)
+    out = torch.empty((n, 8), dtype=torch.int16, device="cuda")
+    lwe.matmul_modq(lwe.SIDE_AS, dev(St), out, n, logq, A=A, seedA=sd, E=dev(E))
+    assert np.array_equal(as_u16(out), O.mul_AS(A_o, St, E, logq))
+    out2 = torch.empty((k, n), dtype=torch.int16, device="cuda")
+    lwe.matmul_modq(lwe.SIDE_SA, dev(S), out2, n, logq, A=A, seedA=sd, E=dev(E2))
+    assert np.array_equal(as_u16(out2), O.mul_SA(S, A_o, E2, logq))
+
+
+@pytest.mark.parametrize("n,count", [(304, 250), (16, 2500), (640, 130)])
+def test_many_regenerated_items_match_oracle(n, count):
+    """Enough row tiles that a warp takes whole tiles (k_mul_as_gen); at n =
+    16 a CTA's range spans more items than it holds tables for."""
+    p, po = params("P640", n=n)
+    ctx = lwe.Ctx(p, max_batch=count)
+    ms = master_seeds(count, seed=n)
+    pk, sk = ctx.empty_pk(count), ctx.empty_sk(count)
+    ctx.keygen(dev(ms), pk, sk)
+    pk_h, sk_h = host(pk), host(sk)
+    for i in list(range(0, count, max(1, count // 40))) + [count - 1]:
+        pk_o, sk_o = O.keygen(po, bytes(ms[i]))
+        assert np.array_equal(pk_h[i], pk_o), i
+        assert np.array_equal(sk_h[i], sk_o), i
+    ctx.close()
