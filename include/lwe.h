@@ -149,11 +149,12 @@ enum {
   LWE_OPT_WARP_HASH_MAX = 7, /* hashing launches (tree hashes H(pk), H(c);
                                 KeyGen seeds; mu, K', seedSE'; the Decaps
                                 key) of at most this many items run with
-                                one Keccak state per warp (the lanes of
-                                the state spread over the threads: lower
+                                ten threads per Keccak state (lower
                                 latency), larger ones with one state per
                                 thread (higher throughput).  -1 (default):
-                                the number of SMs; 0: always per thread   */
+                                8 items per SM, tree hashes while there are
+                                at most 44 1024-byte leaves per SM or one
+                                message per SM; 0: always per thread      */
   LWE_OPT_PDL = 8,           /* 1 (default): the kernels of Encaps / Decaps
                                 are launched with programmatic stream
                                 serialisation (each may start while the
@@ -388,8 +389,9 @@ int lwe_bounds_violations(uint64_t *count, uint32_t *first_site);
  *     under one key per warp (the generator of the noise and of A); iters
  *     a multiple of 4.
  *   LWE_PROBE_KECCAK_WARP: `ctas` CTAs of one warp; each warp applies
- *     Keccak-f[1600] `iters` times to one state spread over its lanes (the
- *     permutation of k_tree_warp).  Work: ctas * iters permutations.
+ *     Keccak-f[1600] `iters` times to one state spread over ten lanes (the
+ *     permutation of k_tree_warp; the warp's other lanes carry the state
+ *     twice more).  Work: ctas * iters permutations.
  * One word per thread is written to sink (device, >= ctas * 512 words) so
  * that the work is kept.  Asynchronous on `stream`; time it with CUDA events
  * there.  LWE_EINVAL for an unknown kind, ctas = 0, or iters not a multiple

@@ -7,15 +7,16 @@
 #pragma once
 #include "common.cuh"
 
-__constant__ uint64_t kKeccakRC[24] = {
-    0x0000000000000001ull, 0x0000000000008082ull, 0x800000000000808Aull,
-    0x8000000080008000ull, 0x000000000000808Bull, 0x0000000080000001ull,
-    0x8000000080008081ull, 0x8000000000008009ull, 0x000000000000008Aull,
-    0x0000000000000088ull, 0x0000000080008009ull, 0x000000008000000Aull,
-    0x000000008000808Bull, 0x800000000000008Bull, 0x8000000000008089ull,
-    0x8000000000008003ull, 0x8000000000008002ull, 0x8000000000000080ull,
-    0x000000000000800Aull, 0x800000008000000Aull, 0x8000000080008081ull,
-    0x8000000000008080ull, 0x0000000080000001ull, 0x8000000080008008ull};
+#define KECCAK_RC \
+  0x0000000000000001ull, 0x0000000000008082ull, 0x800000000000808Aull, \
+  0x8000000080008000ull, 0x000000000000808Bull, 0x0000000080000001ull, \
+  0x8000000080008081ull, 0x8000000000008009ull, 0x000000000000008Aull, \
+  0x0000000000000088ull, 0x0000000080008009ull, 0x000000008000000Aull, \
+  0x000000008000808Bull, 0x800000000000008Bull, 0x8000000000008089ull, \
+  0x8000000000008003ull, 0x8000000000008002ull, 0x8000000000000080ull, \
+  0x000000000000800Aull, 0x800000008000000Aull, 0x8000000080008081ull, \
+  0x8000000000008080ull, 0x0000000080000001ull, 0x8000000080008008ull
+__constant__ uint64_t kKeccakRC[24] = {KECCAK_RC};
 
 // 64-bit rotation; compiles to a pair of funnel shifts.  (Rotations written
 // as multiply-adds to unload the integer ALU pipe were measured slower: more

@@ -169,8 +169,12 @@ struct NoiseRun {
 
 LWE_DEV NoiseRun noise_run_of(const NoiseArgs &a, uint64_t run) {
   NoiseRun x;
-  x.e = (uint32_t)(run / a.runs_per_item);
-  x.r = (uint32_t)(run % a.runs_per_item);
+  if (run >> 32) {
+    x.e = (uint32_t)(run / a.runs_per_item);
+  } else {  // a 32-bit division where it does (the other takes ~100 instructions)
+    x.e = (uint32_t)run / a.runs_per_item;
+  }
+  x.r = (uint32_t)(run - (uint64_t)x.e * a.runs_per_item);
   x.s = 0;
   while (x.s + 1 < a.nout && x.r >= a.out[x.s].runs) {
     x.r -= a.out[x.s].runs;
@@ -205,7 +209,7 @@ LWE_DEV void noise_runs(const NoiseArgs &a, const AesTab &tab, const char *smem,
         if (LWE_BOUNDS(x.e < a.count, 108)) {
           uint32_t rk[44];
           noise_load_rk(a, x.e, rk);
-          mine = aes_ctr_run(tab, rk, a.out[x.s].domain, x.r * NOISE_RUN);
+          mine = aes_ctr_run(tab, rk, a.out[x.s].domain, x.r * a.run);
         }
       }
     }
@@ -222,8 +226,8 @@ LWE_DEV void noise_runs(const NoiseArgs &a, const AesTab &tab, const char *smem,
       uint8_t *base = reinterpret_cast<uint8_t *>(o.base) + (size_t)x.e * o.item_stride;
       // a run lies inside one 256-aligned window of counter indices, whose
       // first two AES rounds are in `win`
-      const uint32_t first = x.r * NOISE_RUN, b0 = first + lane, x0 = (first & 255u) + lane;
-      if (first + NOISE_RUN <= nblk) {
+      const uint32_t first = x.r * a.run, b0 = first + lane, x0 = (first & 255u) + lane;
+      if (a.run == NOISE_RUN && first + NOISE_RUN <= nblk) {
         // full run: two independent blocks in flight per lane
 #pragma unroll
         for (uint32_t jj = 0; jj < NOISE_RUN / 32; jj += 2) {
@@ -234,7 +238,7 @@ LWE_DEV void noise_runs(const NoiseArgs &a, const AesTab &tab, const char *smem,
         }
       } else {
 #pragma unroll 1
-        for (uint32_t b = b0; b < nblk; b += 32)
+        for (uint32_t b = b0; b < min(nblk, first + a.run); b += 32)
           noise_store(smem, o, base, b, aes_ctr_run_block(tab, rk, win, x0 + (b - b0)));
       }
     }
@@ -501,23 +505,45 @@ LWE_DEV void st_le64(uint8_t *p, uint64_t v) {
   for (int b = 0; b < 8; b++) p[b] = (uint8_t)(v >> (8 * b));
 }
 
-// lane t of prefix || 32 bytes, padded: the 32 bytes shifted up one byte,
-// the padding opening byte 1 of lane 4
-LWE_DEV uint64_t prefixed32_lane(uint8_t prefix, const uint8_t *msg32, uint32_t t) {
-  uint64_t v = 0;
-  if (t < 4) v = ld_le64(msg32 + 8 * t) << 8;
-  if (t >= 1 && t <= 4) v |= ld_le64(msg32 + 8 * (t - 1)) >> 56;
-  if (t == 0) v |= prefix;
-  if (t == 4) v |= 0x0600ull;
-  if (t == SHA3_RATE / 8 - 1) v ^= 0x8000000000000000ull;
+// word w of a padded single-block message of 8 nw bytes
+LWE_DEV uint64_t sha3_pad_word(uint32_t w, uint32_t nw) {
+  return (w == nw ? 0x06ull : 0ull) ^ (w == SHA3_RATE / 8 - 1 ? 0x8000000000000000ull : 0ull);
+}
+
+// word w of prefix || 32 bytes, padded: the 32 bytes shifted up one byte,
+// the padding opening byte 1 of word 4
+LWE_DEV uint64_t prefixed32_word(uint8_t prefix, const uint8_t *msg32, uint32_t w) {
+  uint64_t v = sha3_pad_word(w, 4) & ~0xffull;
+  if (w < 4) v |= ld_le64(msg32 + 8 * w) << 8;
+  if (w >= 1 && w <= 4) v |= ld_le64(msg32 + 8 * (w - 1)) >> 56;
+  if (w == 0) v |= prefix;
+  if (w == 4) v |= 0x0600ull;
   return v;
 }
 
-// KeyGen seeds (Alg. 1): warp j of the item's CTA hashes prefix j || ms
-__global__ void __launch_bounds__(96) k_keygen_seeds_warp(KeygenSeedArgs a) {
+// The key schedule of the 16-byte seed held as digest words 0..3 by the
+// threads first .. first + 3, written to rk; the whole warp calls it.
+LWE_DEV void warp_store_schedule(const uint32_t *sT0, uint32_t v, uint32_t first, uint32_t lane,
+                                 uint32_t *out) {
+  uint32_t key[4], rk[44];
+#pragma unroll
+  for (uint32_t i = 0; i < 4; i++) key[i] = tri_shfl(v, first + i);
+  if (lane != first) return;
+  aes_key_expand_global(sT0, key, rk);
+  uint4 *dst = reinterpret_cast<uint4 *>(out);
+#pragma unroll
+  for (int i = 0; i < 11; i++)
+    dst[i] = make_uint4(rk[4 * i], rk[4 * i + 1], rk[4 * i + 2], rk[4 * i + 3]);
+}
+
+// KeyGen seeds (Alg. 1): group j of the item's warp hashes prefix j || ms;
+// four items per CTA
+__global__ void __launch_bounds__(128) k_keygen_seeds_warp(KeygenSeedArgs a) {
   __shared__ uint32_t sT0[256];
   pdl_trigger();
-  for (uint32_t i = threadIdx.x; i < 256; i += blockDim.x) sT0[i] = g_aes_T0[i];
+  const uint32_t e = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  for (uint32_t i = threadIdx.x; i < 256; i += 128) sT0[i] = g_aes_T0[i];
+  const KeccakTri km = keccak_tri(lane);
   __syncthreads();
   pdl_wait();
   const uint32_t e = blockIdx.x, w = threadIdx.x >> 5, lane = threadIdx.x & 31, t = lane % 25;
@@ -527,102 +553,93 @@ __global__ void __launch_bounds__(96) k_keygen_seeds_warp(KeygenSeedArgs a) {
   uint8_t *pk = a.pk + (size_t)e * a.pk_bytes;
   uint8_t *sk = a.sk + (size_t)e * a.sk_bytes;
   uint8_t *ws = a.ws_seeds + 32 * (size_t)e;
-  if (w == 0) {  // seedA
-    if (lane < 2) {
-      st_le64(pk + 8 * lane, v);
-      st_le64(sk + a.sk_pk_off + 8 * lane, v);
-      st_le64(ws + 8 * lane, v);
+  if (lane < 30) {
+    if (km.grp == 0 && r < 4) {  // seedA
+      st_le32(pk + 4 * r, v);
+      st_le32(sk + a.sk_pk_off + 4 * r, v);
+      st_le32(ws + 4 * r, v);
+    } else if (km.grp == 1 && r < 4) {  // seedSE
+      st_le32(ws + 16 + 4 * r, v);
+    } else if (km.grp == 2 && r < 8) {  // z
+      st_le32(sk + a.sk_z_off + 4 * r, v);
     }
-  } else if (w == 1) {  // seedSE and its key schedule
-    if (lane < 2) st_le64(ws + 16 + 8 * lane, v);
-    const uint64_t v1 = shfl64(v, 1);
-    if (lane == 0) {
-      const uint32_t key[4] = {(uint32_t)v, (uint32_t)(v >> 32), (uint32_t)v1, (uint32_t)(v1 >> 32)};
-      uint32_t rk[44];
-      aes_key_expand_global(sT0, key, rk);
-      uint4 *dst = reinterpret_cast<uint4 *>(a.ws_rk + 44 * (size_t)e);
-#pragma unroll
-      for (int i = 0; i < 11; i++)
-        dst[i] = make_uint4(rk[4 * i], rk[4 * i + 1], rk[4 * i + 2], rk[4 * i + 3]);
-    }
-  } else if (lane < 4) {  // z
-    st_le64(sk + a.sk_z_off + 8 * lane, v);
   }
+  warp_store_schedule(sT0, v, 10, lane, a.ws_rk + 44 * (size_t)e);
 }
 
-// Encaps / Decaps derivation (Alg. 4, 5): both warps of the item's CTA
-// hash mu (Encaps), then warp 0 K' = H(pkh || mu) and warp 1
-// seedSE' = H(0x01 || pkh || mu) with its key schedule
-__global__ void __launch_bounds__(64, 1) k_derive_warp(DeriveArgs a) {
+// Encaps / Decaps derivation (Alg. 4, 5): every group hashes mu (Encaps),
+// then group 0 K' = H(pkh || mu) and group 1 seedSE' = H(0x01 || pkh || mu)
+// with its key schedule
+__global__ void __launch_bounds__(128) k_derive_warp(DeriveArgs a) {
   __shared__ uint32_t sT0[256];
+  __shared__ uint64_t sxs[4][9];  // per warp: pkh (4 words) || mu (4 words) || 0
   pdl_trigger();
-  for (uint32_t i = threadIdx.x; i < 256; i += blockDim.x) sT0[i] = g_aes_T0[i];
+  const uint32_t e = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  uint64_t *sx = sxs[threadIdx.x >> 5];
+  for (uint32_t i = threadIdx.x; i < 256; i += 128) sT0[i] = g_aes_T0[i];
+  const KeccakTri km = keccak_tri(lane);
+  if (lane == 8) sx[8] = 0;
   __syncthreads();
   pdl_wait();
-  const uint32_t e = blockIdx.x, w = threadIdx.x >> 5, lane = threadIdx.x & 31, t = lane % 25;
-  const KeccakWarpMap km = keccak_warp_map(lane);
-  const uint32_t nb = a.mu_bytes / 8;  // lanes of mu, 1..4
-  uint64_t *mu64 = reinterpret_cast<uint64_t *>(a.mu + 32 * (size_t)e);
-  uint64_t mu_l = 0;  // lane t < 4: lane t of mu (zero beyond nb)
-  if (a.coins) {
-    const uint64_t v = keccak_f1600_warp(km, prefixed32_lane(0x4D, a.coins + 32 * (size_t)e, t));
-    mu_l = t < nb ? v : 0;
-    if (w == 0 && lane < 4) mu64[lane] = mu_l;
-  } else if (t < nb) {
-    mu_l = mu64[t];
-  }
-  // x = pkh (4 lanes) || mu (4 lanes) || zeros; thread t holds x[t]
+  if (e >= a.count) return;  // the whole warp
+  const uint32_t nb = a.mu_bytes / 8;  // words of mu, 1..4
+  uint32_t *mu = reinterpret_cast<uint32_t *>(a.mu + 32 * (size_t)e);
   const uint8_t *pkh = a.pkh_ptrs ? a.pkh_ptrs[e] + a.pkh_off : a.pkh + (size_t)e * a.pkh_stride;
-  const uint64_t mu_at = shfl64(mu_l, (lane - 4) & 31);
-  const uint64_t x = t < 4 ? ld_le64(pkh + 8 * t) : (t < 8 ? mu_at : 0);
-  if (w == 0) {
-    uint64_t m = x;
-    if (t == 4 + nb) m ^= 0x06ull;
-    if (t == SHA3_RATE / 8 - 1) m ^= 0x8000000000000000ull;
-    const uint64_t v = keccak_f1600_warp(km, m);
-    if (lane < 4) st_le64(a.kprime + 32 * (size_t)e + 8 * lane, v);
-    return;
+  if (lane >= 16 && lane < 20) sx[lane - 16] = ld_le64(pkh + 8 * (lane - 16));
+  uint32_t s[5];
+  uint32_t m = 0;  // thread r < 8: 32-bit word r of mu (zero beyond nb words)
+  if (a.coins) {
+    const uint8_t *coins = a.coins + 32 * (size_t)e;
+    tri_one_block(km, s, [&](uint32_t w) { return prefixed32_word(0x4D, coins, w); });
+    m = tri_digest_word(km, s);
+    if (lane < 8) {
+      if (lane >= 2 * nb) m = 0;
+      mu[lane] = m;
+    }
+  } else if (lane < 2 * nb) {
+    m = mu[lane];
   }
-  const uint64_t xp = shfl64(x, (lane + 31) & 31);  // x[t - 1]
-  uint64_t m = t == 0 ? (0x01ull | (x << 8)) : ((xp >> 56) | (x << 8));
-  if (t == 4 + nb) m ^= 0x0600ull;
-  if (t == SHA3_RATE / 8 - 1) m ^= 0x8000000000000000ull;
-  const uint64_t v = keccak_f1600_warp(km, m);
-  if (lane < 2) st_le64(a.seeds + 32 * (size_t)e + 8 * lane, v);
-  const uint64_t v1 = shfl64(v, 1);
-  if (lane == 0) {
-    const uint32_t key[4] = {(uint32_t)v, (uint32_t)(v >> 32), (uint32_t)v1, (uint32_t)(v1 >> 32)};
-    uint32_t rk[44];
-    aes_key_expand_global(sT0, key, rk);
-    uint4 *dst = reinterpret_cast<uint4 *>(a.rk + 44 * (size_t)e);
-#pragma unroll
-    for (int i = 0; i < 11; i++)
-      dst[i] = make_uint4(rk[4 * i], rk[4 * i + 1], rk[4 * i + 2], rk[4 * i + 3]);
+  if (lane < 8) reinterpret_cast<uint32_t *>(sx + 4)[lane] = m;
+  __syncwarp();
+  // the two messages: x || padding, and the same one byte later after 0x01
+  const bool enc = km.grp == 1;
+  tri_one_block(km, s, [&](uint32_t w) -> uint64_t {
+    const uint64_t x = sx[min(w, 8u)], pad = sha3_pad_word(w, 4 + nb);
+    if (!enc) return x ^ pad;
+    const uint64_t xp = w == 0 ? 0ull : sx[min(w - 1, 8u)];
+    return (w == 0 ? 0x01ull : xp >> 56) ^ (x << 8) ^ (pad & ~0xffull) ^
+           (w == 4 + nb ? 0x0600ull : 0ull);
+  });
+  const uint32_t v = tri_digest_word(km, s), r = km.r;
+  if (lane < 30) {
+    if (km.grp == 0 && r < 8) st_le32(a.kprime + 32 * (size_t)e + 4 * r, v);
+    if (km.grp == 1 && r < 4) st_le32(a.seeds + 32 * (size_t)e + 4 * r, v);
   }
+  warp_store_schedule(sT0, v, 10, lane, a.rk + 44 * (size_t)e);
 }
 
 // Decaps key (Alg. 5): K = H(K' || H(c)) when the re-encryption matched,
 // else H(z || H(c)); one warp per item
-__global__ void __launch_bounds__(32) k_final_key_warp(FinalKeyArgs a) {
+__global__ void __launch_bounds__(128) k_final_key_warp(FinalKeyArgs a) {
   pdl_trigger();
+  const uint32_t e = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const KeccakTri km = keccak_tri(lane);
   pdl_wait();
-  const uint32_t e = blockIdx.x, lane = threadIdx.x, t = lane % 25;
-  const KeccakWarpMap km = keccak_warp_map(lane);
+  if (e >= a.count) return;  // the whole warp
   const uint32_t f = a.flags[e];
   const uint64_t keep = (uint64_t)0 - (uint64_t)(((f | (0u - f)) >> 31) ^ 1u);
-  uint64_t m = 0;
-  if (t < 4) {
-    const uint64_t *kp = reinterpret_cast<const uint64_t *>(a.kprime + 32 * (size_t)e);
-    const uint64_t *z =
-        reinterpret_cast<const uint64_t *>(a.z_ptrs ? a.z_ptrs[e] + a.z_off : a.z);
-    m = (kp[t] & keep) | (z[t] & ~keep);
-  } else if (t < 8) {
-    m = reinterpret_cast<const uint64_t *>(a.hc + 32 * (size_t)e)[t - 4];
-  }
-  if (t == 8) m ^= 0x06ull;
-  if (t == SHA3_RATE / 8 - 1) m ^= 0x8000000000000000ull;
-  const uint64_t v = keccak_f1600_warp(km, m);
-  if (lane < 4) st_le64(a.K + 32 * (size_t)e + 8 * lane, v);
+  const uint64_t *kp = reinterpret_cast<const uint64_t *>(a.kprime + 32 * (size_t)e);
+  const uint64_t *z = reinterpret_cast<const uint64_t *>(a.z_ptrs ? a.z_ptrs[e] + a.z_off : a.z);
+  const uint64_t *hc = reinterpret_cast<const uint64_t *>(a.hc + 32 * (size_t)e);
+  uint32_t s[5];
+  tri_one_block(km, s, [&](uint32_t w) -> uint64_t {
+    uint64_t v = sha3_pad_word(w, 8);
+    if (w < 4) v ^= (kp[w] & keep) | (z[w] & ~keep);
+    else if (w < 8) v ^= hc[w - 4];
+    return v;
+  });
+  const uint32_t v = tri_digest_word(km, s);
+  if (lane < 8) st_le32(a.K + 32 * (size_t)e + 4 * lane, v);
 }
 
 // Tree hash: tpi threads per message compute its 1024-byte-chunk digests
@@ -901,66 +918,75 @@ __global__ void __maxnreg__(96) k_tree_dense(TreeArgs a) {
   }
 }
 
-// Tree hash with one Keccak state per warp (keccak_warp.cuh), for launches
-// of few messages, where one state per thread would leave the GPU idle
-// behind a chain of sequential permutations.  A thread-block cluster of Q
-// CTAs (W warps each, on Q SMs, so that few warps share an SM's shuffle
-// unit) takes one message: warp w of CTA q hashes chunks qW + w, qW + w +
-// QW, ... and stores each digest in the shared memory of the cluster's
-// first CTA, whose warp 0 then hashes the digests (the root) and, for
-// Encaps, derives the key.
-LWE_DEV void st_cluster_u64(uint32_t addr, uint64_t v) {
-  asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
-}
-
-// The end of a tree hash on one warp (v: this lane of the root's final
-// state, lanes 0..3 the digest): digest mode stores H into out (and out2);
-// Encaps mode derives K = H(K' || H(c)) (Alg. 4), one 64-byte block.
-LWE_DEV void tree_warp_out(const TreeArgs &a, uint32_t e, const KeccakWarpMap &km, uint32_t lane,
-                           uint64_t v) {
-  const uint32_t t = lane % 25;
-  uint8_t *out;
+// The end of a tree hash (s: the final state of each group's root, message e
+// of the group if `in`): digest mode stores H into out (and out2); Encaps mode
+// derives K = H(K' || H(c)) (Alg. 4), one 64-byte block.
+LWE_DEV void tree_tri_out(const TreeArgs &a, uint32_t e, bool in, const KeccakTri &km,
+                          uint32_t lane, uint32_t s[5]) {
+  uint32_t v = tri_digest_word(km, s);
+  const bool st = in && lane < 30 && km.r < 8;
   if (a.mode == TREE_DIGEST) {
-    if (a.out2 && lane < 4) {
-      uint8_t *o2 = a.out2 + (size_t)e * a.out2_stride + 8 * lane;
-      for (int b = 0; b < 8; b++) o2[b] = (uint8_t)(v >> (8 * b));
-    }
-    out = a.out + (size_t)e * a.out_stride;
-  } else {
-    const uint64_t hc = shfl64(v, (lane - 4) & 31);  // lanes 4..7 take the digest
-    uint64_t w = 0;
-    if (t < 4) w = reinterpret_cast<const uint64_t *>(a.kprime + 32 * (size_t)e)[t];
-    else if (t < 8) w = hc;
-    if (t == 8) w ^= 0x06;
-    if (t == SHA3_RATE / 8 - 1) w ^= 0x8000000000000000ull;
-    v = keccak_f1600_warp(km, w);
-    out = a.out + 32 * (size_t)e;
+    if (st) st_le32(a.out + (size_t)e * a.out_stride + 4 * km.r, v);
+    if (st && a.out2) st_le32(a.out2 + (size_t)e * a.out2_stride + 4 * km.r, v);
+    return;
   }
-  if (lane < 4)
-    for (int b = 0; b < 8; b++) out[8 * lane + b] = (uint8_t)(v >> (8 * b));
+  uint64_t hc[4];
+#pragma unroll
+  for (uint32_t i = 0; i < 4; i++)
+    hc[i] = (uint64_t)tri_shfl(v, 10 * km.grp + 2 * i) |
+            ((uint64_t)tri_shfl(v, 10 * km.grp + 2 * i + 1) << 32);
+  const uint64_t *kp = reinterpret_cast<const uint64_t *>(a.kprime + 32 * (size_t)(in ? e : 0));
+  tri_one_block(km, s, [&](uint32_t w) -> uint64_t {
+    uint64_t x = sha3_pad_word(w, 8);
+    if (w < 4) x ^= kp[w];
+#pragma unroll
+    for (uint32_t i = 0; i < 4; i++) x ^= w == 4 + i ? hc[i] : 0ull;
+    return x;
+  });
+  v = tri_digest_word(km, s);
+  if (st) st_le32(a.out + 32 * (size_t)e + 4 * km.r, v);
 }
 
-__global__ void __launch_bounds__(TREE_WARP_MAX_THREADS, 1) k_tree_warp(TreeArgs a) {
+// Tree hash with three Keccak states per warp (keccak_warp.cuh), for launches
+// whose leaves leave the SMs so empty that a permutation's latency counts.  A
+// thread-block cluster of Q CTAs (W warps each) takes one message: warp w of
+// CTA q hashes chunks 3 (qW + w) .. + 2, then those 3 QW further on, and
+// stores each digest in the shared memory of the cluster's first CTA, whose
+// warp 0 then hashes the digests (the root) and, for Encaps, derives the key.
+LWE_DEV void st_cluster_u32(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+
+__global__ void __maxnreg__(112) k_tree_warp(TreeArgs a) {
   extern __shared__ uint64_t sdig[];  // [m][4], used in the cluster's first CTA
   pdl_trigger();
-  pdl_wait();
   uint32_t q, nq;
   asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(q));
   asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(nq));
   const uint32_t e = blockIdx.x / nq, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t nw = blockDim.x >> 5;
-  const KeccakWarpMap km = keccak_warp_map(lane);
+  const KeccakTri km = keccak_tri(lane);
+  // every CTA of the cluster has started before any stores into the first
+  if (nq > 1) cluster_barrier();
+  pdl_wait();
   const uint8_t *msg = a.msg_ptrs ? a.msg_ptrs[e] : a.msgs + (size_t)e * a.stride;
   const uint32_t dig0 = cluster_map(sdig, 0);
-  for (uint32_t c = q * nw + warp; c < a.m; c += nq * nw) {
-    const uint32_t off = c * LWE_TREE_CHUNK;
-    const uint64_t v =
-        sha3_256_warp_chunk(km, msg + off, min((uint32_t)LWE_TREE_CHUNK, a.len - off), lane);
-    if (lane < 4) st_cluster_u64(dig0 + 8 * (4 * c + lane), v);
+  const uint32_t len = a.len;
+  const uint32_t mc = (len + LWE_TREE_CHUNK - 1) / LWE_TREE_CHUNK;
+  uint32_t s[5];
+  for (uint32_t c0 = 3 * (q * nw + warp); c0 < mc; c0 += 3 * nq * nw) {
+    const uint32_t c = c0 + km.grp, off = c * LWE_TREE_CHUNK;
+    const bool in = c < mc && LWE_BOUNDS(off < len, 106);
+    sha3_256_tri<true>(km, msg + (in ? off : 0),
+                       in ? min((uint32_t)LWE_TREE_CHUNK, len - off) : 0u, s);
+    const uint32_t v = tri_digest_word(km, s);
+    if (in && lane < 30 && km.r < 8) st_cluster_u32(dig0 + 4 * (8 * c + km.r), v);
   }
-  cluster_barrier();  // every digest is in the first CTA's shared memory
+  if (nq > 1) cluster_barrier();  // every digest is in the first CTA's shared memory
+  else __syncthreads();
   if (q != 0 || warp != 0) return;
-  tree_warp_out(a, e, km, lane, sha3_256_warp_mem(km, sdig, 32 * a.m, lane));
+  sha3_256_tri<false>(km, reinterpret_cast<const uint8_t *>(sdig), km.grp ? 0u : 32 * mc, s);
+  tree_tri_out(a, e, km.grp == 0, km, lane, s);
 }
 
 // Tree hash of long messages (more than 32 chunks: ciphertexts and public
@@ -989,14 +1015,36 @@ __global__ void __launch_bounds__(256) k_tree_leaves(TreeArgs a) {
   d[1] = make_uint4((uint32_t)s[2], (uint32_t)(s[2] >> 32), (uint32_t)s[3], (uint32_t)(s[3] >> 32));
 }
 
+// The leaves with three states per warp, where one thread per leaf would leave
+// the SMs behind a few warps' 5.6 us permutations.
+__global__ void __launch_bounds__(64) k_tree_leaves_tri(TreeArgs a) {
+  pdl_trigger();
+  const uint32_t lane = threadIdx.x & 31;
+  const KeccakTri km = keccak_tri(lane);
+  const uint64_t L = 3ull * (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) + km.grp;
+  pdl_wait();
+  const uint32_t e = (uint32_t)(L / a.m), off = (uint32_t)(L % a.m) * LWE_TREE_CHUNK;
+  const bool in = L < (uint64_t)a.count * a.m &&
+                  LWE_BOUNDS(off < a.len && 4 * (L + 1) <= a.dig_words, 114);
+  const uint8_t *msg = !in ? nullptr : a.msg_ptrs ? a.msg_ptrs[e] : a.msgs + (size_t)e * a.stride;
+  uint32_t s[5];
+  sha3_256_tri<true>(km, msg + (in ? off : 0), in ? min((uint32_t)LWE_TREE_CHUNK, a.len - off) : 0u,
+                     s);
+  const uint32_t v = tri_digest_word(km, s);
+  if (in && lane < 30 && km.r < 8) reinterpret_cast<uint32_t *>(a.dig + 4 * L)[km.r] = v;
+}
+
 __global__ void __launch_bounds__(64) k_tree_roots(TreeArgs a) {
   pdl_trigger();
+  const uint32_t lane = threadIdx.x & 31;
+  const KeccakTri km = keccak_tri(lane);
+  const uint32_t e = 3 * (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) + km.grp;
   pdl_wait();
-  const uint32_t e = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (e >= a.count) return;  // the whole warp
-  const KeccakWarpMap km = keccak_warp_map(lane);
-  if (!LWE_BOUNDS(4ull * (e + 1) * a.m <= a.dig_words, 115)) return;
-  tree_warp_out(a, e, km, lane, sha3_256_warp_mem(km, a.dig + 4ull * e * a.m, 32 * a.m, lane));
+  const bool in = e < a.count && LWE_BOUNDS(4ull * (e + 1) * a.m <= a.dig_words, 115);
+  uint32_t s[5];
+  sha3_256_tri<false>(km, reinterpret_cast<const uint8_t *>(a.dig + (in ? 4ull * e * a.m : 0)),
+                      in ? 32 * a.m : 0u, s);
+  tree_tri_out(a, e, in, km, lane, s);
 }
 
 __global__ void __launch_bounds__(128) k_final_key(FinalKeyArgs a) {
@@ -1188,10 +1236,21 @@ __global__ void __launch_bounds__(512, 1) k_probe_aes_run(uint32_t iters, uint32
 }
 
 __global__ void __launch_bounds__(32) k_probe_keccak_warp(uint32_t iters, uint32_t *sink) {
+  __shared__ uint32_t sh[2][25];
   const uint32_t lane = threadIdx.x, t = lane % 25;
-  const KeccakWarpMap km = keccak_warp_map(lane);
-  uint64_t v = ((uint64_t)blockIdx.x << 32) ^ (uint64_t)(t * 0x9E3779B9u);
-  for (uint32_t it = 0; it < iters; it++) v = keccak_f1600_warp(km, v);
+  const KeccakTri km = keccak_tri(lane);
+  uint32_t s[5];
+#pragma unroll
+  for (uint32_t i = 0; i < 5; i++)
+    s[i] = tri_half(((uint64_t)blockIdx.x << 32) ^ (uint64_t)(tri_lane(km, i) * 0x9E3779B9u), km.h);
+  for (uint32_t it = 0; it < iters; it++) keccak_f1600_tri(km, s);
+  if (lane < 10)
+#pragma unroll
+    for (uint32_t i = 0; i < 5; i++) sh[km.h][tri_lane(km, i)] = s[i];
+  __syncwarp();
+  uint64_t v = 0;
+  for (uint32_t b = 0; b < 32; b++)
+    v |= ((uint64_t)((sh[0][t] >> b) & 1u) << (2 * b)) | ((uint64_t)((sh[1][t] >> b) & 1u) << (2 * b + 1));
   sink[32 * blockIdx.x + lane] = (uint32_t)(v ^ (v >> 32));
 }
 
@@ -1328,7 +1387,7 @@ void launch_noise_table(const NoiseArgs &a, int8_t *out, cudaStream_t st) {
 }
 
 void launch_noise(const NoiseArgs &a, int num_sms, cudaStream_t st) {
-  const int g = grid_for((uint64_t)a.count * a.runs_per_item, 16, num_sms);
+  const int g = grid_for((uint64_t)a.count * a.runs_per_item, a.run == NOISE_RUN ? 16 : 1, num_sms);
   launch_k(k_noise, g, 512, NOISE_SMEM_BYTES, st, a);
 }
 
@@ -1430,7 +1489,7 @@ void launch_mul_sa(const MulSaArgs &a, uint32_t items, bool fused, bool cmp, int
 
 void launch_keygen_seeds(const KeygenSeedArgs &a, uint32_t warp_max, cudaStream_t st) {
   if (a.count <= warp_max) {
-    launch_k(k_keygen_seeds_warp, a.count, 96, 0, st, a);
+    launch_k(k_keygen_seeds_warp, (a.count + 3) / 4, 128, 0, st, a);
     return;
   }
   launch_k(k_keygen_seeds, (a.count + 63) / 64, 64, 0, st, a);
@@ -1438,7 +1497,7 @@ void launch_keygen_seeds(const KeygenSeedArgs &a, uint32_t warp_max, cudaStream_
 
 void launch_derive(const DeriveArgs &a, uint32_t warp_max, cudaStream_t st) {
   if (a.count <= warp_max) {
-    launch_k(k_derive_warp, a.count, 64, 0, st, a);
+    launch_k(k_derive_warp, (a.count + 3) / 4, 128, 0, st, a);
     return;
   }
   launch_k(k_derive, (a.count + 31) / 32, 64, 0, st, a);
@@ -1449,15 +1508,23 @@ void launch_derive(const DeriveArgs &a, uint32_t warp_max, cudaStream_t st) {
 // of digests per CTA.
 void launch_tree(TreeArgs &a, int num_sms, uint32_t warp_max, cudaStream_t st) {
   a.m = (a.len + LWE_TREE_CHUNK - 1) / LWE_TREE_CHUNK;
+  const uint32_t sms = num_sms > 0 ? (uint32_t)num_sms : 1u;
+  const bool dig_fits = a.dig && (uint64_t)a.count * a.m * 4 <= a.dig_words;
   if (a.count <= warp_max) {
-    // about four warps per SM: chunks over a cluster of up to 8 CTAs
-    const uint32_t q = std::max<uint32_t>(1, std::min<uint32_t>(8, (a.m + 3) / 4));
-    const uint32_t w = std::min<uint32_t>((a.m + q - 1) / q, TREE_WARP_MAX_THREADS / 32);
+    if (a.m > 96 && dig_fits) {
+      // more leaves than a cluster of 8 CTAs runs at full speed
+      const uint64_t warps = ((uint64_t)a.count * a.m + 2) / 3;
+      launch_k(k_tree_leaves_tri, (uint32_t)((warps + 1) / 2), 64, 0, st, a);
+      launch_k(k_tree_roots, (a.count + 5) / 6, 64, 0, st, a);
+      return;
+    }
+    // up to 8 warps (24 leaves) per CTA, long messages over a cluster of up to 8
+    const uint32_t q = std::max<uint32_t>(1, std::min<uint32_t>(8, (a.m + 23) / 24));
+    const uint32_t w = std::min<uint32_t>((a.m + 3 * q - 1) / (3 * q), TREE_WARP_MAX_THREADS / 32);
     launch_k_cluster(k_tree_warp, a.count * q, 32 * w, (size_t)a.m * 32, st, q, a);
     return;
   }
-  const uint32_t sms = num_sms > 0 ? (uint32_t)num_sms : 1u;
-  if (a.m > 32 && a.dig && (uint64_t)a.count * a.m * 4 <= a.dig_words) {
+  if (a.m > 32 && dig_fits) {
     // long messages: every leaf on its own thread, then one warp per root,
     // once k_tree (below: one thread per message runs its root) would have
     // root chains of more than 128 chunks (31+ sequential permutations) or
@@ -1471,7 +1538,7 @@ void launch_tree(TreeArgs &a, int num_sms, uint32_t warp_max, cudaStream_t st) {
       const uint64_t leaves = (uint64_t)a.count * a.m;
       const uint32_t lt = leaves >= (uint64_t)sms * 1024 ? 256u : 64u;
       launch_k(k_tree_leaves, (uint32_t)((leaves + lt - 1) / lt), lt, 0, st, a);
-      launch_k(k_tree_roots, (a.count + 1) / 2, 64, 0, st, a);
+      launch_k(k_tree_roots, (a.count + 5) / 6, 64, 0, st, a);
       return;
     }
   }
@@ -1528,7 +1595,7 @@ void launch_tree(TreeArgs &a, int num_sms, uint32_t warp_max, cudaStream_t st) {
 
 void launch_final_key(const FinalKeyArgs &a, uint32_t warp_max, cudaStream_t st) {
   if (a.count <= warp_max) {
-    launch_k(k_final_key_warp, a.count, 32, 0, st, a);
+    launch_k(k_final_key_warp, (a.count + 3) / 4, 128, 0, st, a);
     return;
   }
   launch_k(k_final_key, (a.count + 127) / 128, 128, 0, st, a);

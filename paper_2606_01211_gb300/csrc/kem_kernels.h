@@ -114,6 +114,7 @@ struct DeriveArgs {
   uint8_t *kprime;       // 32 per item
   uint8_t *seeds;        // 32-byte slot per item, seedSE' in the first 16
   uint32_t *rk;          // 44 round-key words of seedSE' per item
+  uint32_t *flags;       // Decaps: the items' mismatch flags, cleared here; or NULL
   uint32_t count, mu_bytes;
 };
 
@@ -130,6 +131,7 @@ struct TreeArgs {
   const uint8_t *const *msg_ptrs;
   uint64_t stride;
   uint32_t len, count;
+  uint32_t tail_len;     // length of the last message if nonzero, at most len (k_tree_warp only)
   uint32_t m;            // leaves per message
   uint32_t tpi;          // threads per message (power of two <= 256)
   uint32_t ipc;          // messages per CTA

@@ -220,9 +220,21 @@ cudaEvent_t take_event(lwe_ctx *c) {
   return e;
 }
 
-// hashing launches of at most this many items use one Keccak state per warp
+// Hashing launches of at most this many items run ten threads per Keccak
+// state (keccak_warp.cuh) instead of one, LWE_OPT_WARP_HASH_MAX if set.  By
+// default single-block hashes do up to 8 per SM: a permutation then takes ~2 us
+// against 5.6, and beyond about 12 warps per SM the shuffles close the gap.
 uint32_t warp_hash_max(const lwe_ctx *c) {
-  return c->tree_warp_max < 0 ? (uint32_t)c->num_sms : (uint32_t)c->tree_warp_max;
+  return c->tree_warp_max < 0 ? 8u * (uint32_t)c->num_sms : (uint32_t)c->tree_warp_max;
+}
+
+// Tree hashes of m chunks: by default while there are at most 44 leaves per SM
+// (15 warps, one wave of k_tree_warp: 777 messages of 11 chunks, 56 per SM, took
+// 95 us in two waves against 68 with one thread per leaf), and for one short
+// message per SM.
+uint32_t tree_warp_max(int num_sms, uint32_t len) {
+  const uint32_t m = (len + LWE_TREE_CHUNK - 1) / LWE_TREE_CHUNK, sms = (uint32_t)num_sms;
+  return std::max(44u * sms / m, m <= 128 ? sms : 1u);
 }
 
 struct LaunchScope {
@@ -297,8 +309,7 @@ NoiseArgs noise_args(const lwe_ctx *c, uint32_t count) {
 
 NoiseOut noise_out(void *base, uint64_t item_stride, uint32_t nsamples, uint32_t domain,
                    uint32_t fmt) {
-  const uint32_t nblk = (nsamples + 7) / 8;
-  return NoiseOut{base, item_stride, nsamples, domain, fmt, (nblk + NOISE_RUN - 1) / NOISE_RUN};
+  return NoiseOut{base, item_stride, nsamples, domain, fmt, 0};
 }
 
 void noise_finish(NoiseArgs &a) {
@@ -784,7 +795,7 @@ int lwe_keygen(lwe_ctx *c, const uint8_t *seeds, uint32_t count, uint8_t *pk, ui
   na.nout = 2;
   na.out[0] = noise_out(sk, skb, 8 * n, 1, NOISE_I8);           // S^T, row-major 8 x n
   na.out[1] = noise_out(c->ep8, 8ull * n, 8 * n, 2, NOISE_I8);  // E, n x 8
-  noise_finish(na);
+  noise_finish(na, c->num_sms);
   LAUNCH(c, KID_NOISE, st, launch_noise(na, c->num_sms, st));
 
   if (A_out)
@@ -878,7 +889,6 @@ int lwe_decaps(lwe_ctx *c, const uint8_t *sk, const uint16_t *A, const uint8_t *
   const uint8_t *pkh = z + 32;
   const uint8_t *pk = pkh + 32;
 
-  CUDA_TRY(cudaMemsetAsync(c->flags, 0, 4 * (size_t)count, st));
   // H(c) does not depend on the re-encryption: it runs on the side stream,
   // overlapping the re-encryption, and joins before the key selection (the
   // tensor path's limbs go first on that stream)
@@ -900,6 +910,7 @@ int lwe_decaps(lwe_ctx *c, const uint8_t *sk, const uint16_t *A, const uint8_t *
   DecryptArgs dca = decrypt_args(c, ct, reinterpret_cast<const int8_t *>(sk), nullptr);
   LAUNCH(c, KID_DECRYPT, st, launch_decrypt(dca, count, st));
   DeriveArgs da = derive_args(c, nullptr, pkh, count);
+  da.flags = c->flags;
   LAUNCH(c, KID_DERIVE, st, launch_derive(da, warp_hash_max(c), st));
   rc = run_encrypt(c, pk, A, count, const_cast<uint8_t *>(ct), true, st, nullptr, limbs_from);
   if (rc) return rc;
@@ -958,7 +969,6 @@ int lwe_decaps_multi(lwe_ctx *c, const uint8_t *const *sk_ptrs, const uint16_t *
   const lwe_params &p = c->p;
   const uint32_t n = p.n;
   const size_t ctb = ct_bytes(p);
-  CUDA_TRY(cudaMemsetAsync(c->flags, 0, 4 * (size_t)count, st));
   CUDA_TRY(cudaEventRecord(c->ev_fork, st));
   cudaStream_t ss = side_stream(c, st);
   CUDA_TRY(cudaStreamWaitEvent(ss, c->ev_fork, 0));
@@ -1628,7 +1638,7 @@ int lwe_pp_ctx_destroy(lwe_pp_ctx *c) {
   cudaGetDevice(&prev);
   cudaSetDevice(c->device);
   cudaDeviceSynchronize();
-  cudaFree(c->ws);
+  pp_ctx_free(c);
   cudaSetDevice(prev);
   delete c;
   return LWE_OK;

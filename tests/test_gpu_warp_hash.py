@@ -1,0 +1,34 @@
+"""The tree hash with ten threads per Keccak state (k_tree_warp, and
+k_tree_leaves_tri + k_tree_roots for long messages) against hashlib, through
+KeyGen's H(pk): messages of one chunk, of chunk counts that do and do not
+divide by the three states of a warp, of more than one CTA, and of more than
+96 chunks; one item and several."""
+import hashlib
+
+import numpy as np
+import pytest
+import torch
+
+from gpu_util import dev, host, lwe, master_seeds, params
+
+pytestmark = pytest.mark.gpu
+
+
+def _tree(msg: bytes) -> bytes:
+    leaves = [hashlib.sha3_256(msg[i:i + 1024]).digest() for i in range(0, len(msg), 1024)]
+    return hashlib.sha3_256(b"".join(leaves)).digest()
+
+
+@pytest.mark.parametrize("n,count", [(16, 1), (16, 700), (64, 5), (128, 2), (640, 7), (1344, 4),
+                                     (1600, 1), (4096, 3), (6208, 1), (6208, 5), (10240, 2)])
+def test_key_hash_matches_hashlib(n, count):
+    torch.cuda.set_device(0)
+    p, _ = params("P640", n=n)
+    ctx = lwe.Ctx(p, max_batch=count)
+    pk, sk = ctx.empty_pk(count), ctx.empty_sk(count)
+    ctx.keygen(dev(master_seeds(count, seed=n)), pk, sk)
+    pk_h, sk_h = host(pk), host(sk)
+    for i in range(0, count, max(1, count // 16)):
+        got = sk_h[i, 8 * n + 32:8 * n + 64].tobytes()
+        assert got == _tree(pk_h[i].tobytes()), i
+    ctx.close()
