@@ -260,9 +260,11 @@ __global__ void __launch_bounds__(512, 1) k_noise(NoiseArgs a) {
   __syncthreads();
   pdl_wait();
   const AesTab tab = aes_tab(sT);
+  // large calls: a CTA's warps take consecutive runs (mostly one item's);
+  // small ones: consecutive runs go to different SMs
+  const uint64_t nw = blockDim.x >> 5, w = threadIdx.x >> 5;
   noise_runs(a, tab, reinterpret_cast<const char *>(sT),
-             (uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5),
-             (uint64_t)gridDim.x * (blockDim.x >> 5));
+             a.run == NOISE_RUN ? blockIdx.x * nw + w : w * gridDim.x + blockIdx.x, gridDim.x * nw);
 }
 
 LWE_BOUNDS_READER(lwe_bounds_read_kem)
@@ -435,6 +437,7 @@ __global__ void __launch_bounds__(64) k_derive(DeriveArgs a) {
   if (e >= a.count) return;
   uint64_t s[25];
   uint64_t *mu64 = reinterpret_cast<uint64_t *>(a.mu + 32 * (size_t)e);
+  if (a.flags && w == 0) a.flags[e] = 0;
   const uint32_t nb = a.mu_bytes / 8;  // lanes of mu, 1..4
   uint64_t x[8];                       // pkh (4 lanes) || mu (nb lanes) || zeros
   if (a.coins) {
@@ -486,11 +489,10 @@ __global__ void __launch_bounds__(64) k_derive(DeriveArgs a) {
 }
 
 // ---------------------------------------------------------------------------
-// The same hashes with one Keccak state per warp (keccak_warp.cuh), for
-// launches of few items: one permutation then takes one warp ~1.5-2.7 us
-// instead of one thread ~5.6 us, and independent hashes of an item run in
-// different warps.  Thread t builds lane t of the padded single-block
-// message; lanes 0..3 of the result are the digest.
+// The same hashes with ten threads per Keccak state (keccak_warp.cuh), for
+// launches of few items: one permutation then takes ~2 us instead of one
+// thread's ~5.6 us, and the independent hashes of an item run side by side in
+// one warp.
 // ---------------------------------------------------------------------------
 LWE_DEV uint64_t ld_le64(const uint8_t *p) {
   if ((reinterpret_cast<uintptr_t>(p) & 7) == 0) return *reinterpret_cast<const uint64_t *>(p);
@@ -500,9 +502,13 @@ LWE_DEV uint64_t ld_le64(const uint8_t *p) {
   return v;
 }
 
-LWE_DEV void st_le64(uint8_t *p, uint64_t v) {
+LWE_DEV void st_le32(uint8_t *p, uint32_t v) {
+  if ((reinterpret_cast<uintptr_t>(p) & 3) == 0) {
+    *reinterpret_cast<uint32_t *>(p) = v;
+  } else {
 #pragma unroll
-  for (int b = 0; b < 8; b++) p[b] = (uint8_t)(v >> (8 * b));
+    for (int b = 0; b < 4; b++) p[b] = (uint8_t)(v >> (8 * b));
+  }
 }
 
 // word w of a padded single-block message of 8 nw bytes
@@ -546,10 +552,12 @@ __global__ void __launch_bounds__(128) k_keygen_seeds_warp(KeygenSeedArgs a) {
   const KeccakTri km = keccak_tri(lane);
   __syncthreads();
   pdl_wait();
-  const uint32_t e = blockIdx.x, w = threadIdx.x >> 5, lane = threadIdx.x & 31, t = lane % 25;
-  const KeccakWarpMap km = keccak_warp_map(lane);
-  const uint8_t prefix = w == 0 ? 0x41 : (w == 1 ? 0x53 : 0x5A);
-  const uint64_t v = keccak_f1600_warp(km, prefixed32_lane(prefix, a.ms + 32 * (size_t)e, t));
+  if (e >= a.count) return;  // the whole warp
+  const uint8_t prefix = km.grp == 0 ? 0x41 : (km.grp == 1 ? 0x53 : 0x5A);
+  const uint8_t *ms = a.ms + 32 * (size_t)e;
+  uint32_t s[5];
+  tri_one_block(km, s, [&](uint32_t w) { return prefixed32_word(prefix, ms, w); });
+  const uint32_t v = tri_digest_word(km, s), r = km.r;
   uint8_t *pk = a.pk + (size_t)e * a.pk_bytes;
   uint8_t *sk = a.sk + (size_t)e * a.sk_bytes;
   uint8_t *ws = a.ws_seeds + 32 * (size_t)e;

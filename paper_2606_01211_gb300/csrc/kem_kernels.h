@@ -10,10 +10,13 @@
 
 enum { NOISE_I8 = 0, NOISE_BF16 = 1 };
 
-// Noise streams are cut into runs of NOISE_RUN consecutive counter blocks;
-// one warp generates one run (4 blocks per lane), so one item's round keys
-// serve a whole warp and the stores of a warp are contiguous.
+// Noise streams are cut into runs of consecutive counter blocks; one warp
+// generates one run, so one item's round keys serve a whole warp and the
+// stores of a warp are contiguous.  Batches use runs of NOISE_RUN (4 blocks
+// per lane, which share the window constants); calls whose runs would not
+// fill the SMs' warps use runs of NOISE_RUN_SMALL, dealt out over the SMs.
 #define NOISE_RUN 128
+#define NOISE_RUN_SMALL 32
 static_assert(256 % NOISE_RUN == 0, "a noise run lies inside one 256-block counter window");
 
 struct NoiseOut {
@@ -22,7 +25,7 @@ struct NoiseOut {
   uint32_t nsamples;     // samples per item, sample k from word k%8 of block k/8
   uint32_t domain;       // counter-block domain
   uint32_t fmt;          // NOISE_I8 or NOISE_BF16
-  uint32_t runs;         // ceil(ceil(nsamples / 8) / NOISE_RUN)
+  uint32_t runs;         // ceil(ceil(nsamples / 8) / run)
 };
 
 struct NoiseArgs {
@@ -30,7 +33,8 @@ struct NoiseArgs {
   uint32_t count;
   uint32_t nout;
   uint32_t runs_per_item;
-  uint32_t pad0, pad1, pad2;
+  uint32_t run;          // blocks per run
+  uint32_t pad1, pad2;
   NoiseOut out[3];
   uint32_t T[16];        // CDF table, entries >= clip set to 0x7FFF
   const uint4 *tab_img;  // the sampler table for T as k_noise_table writes it

@@ -312,9 +312,19 @@ NoiseOut noise_out(void *base, uint64_t item_stride, uint32_t nsamples, uint32_t
   return NoiseOut{base, item_stride, nsamples, domain, fmt, 0};
 }
 
-void noise_finish(NoiseArgs &a) {
-  a.runs_per_item = 0;
-  for (uint32_t s = 0; s < a.nout; s++) a.runs_per_item += a.out[s].runs;
+// Cuts the streams into runs: short ones while all of them fit two rounds of
+// the SMs' 16 warps (one request: 12 -> 4.5 us at n = 1344), else NOISE_RUN.
+void noise_finish(NoiseArgs &a, int num_sms) {
+  a.run = NOISE_RUN_SMALL;
+  for (;;) {
+    a.runs_per_item = 0;
+    for (uint32_t s = 0; s < a.nout; s++) {
+      a.out[s].runs = ((a.out[s].nsamples + 7) / 8 + a.run - 1) / a.run;
+      a.runs_per_item += a.out[s].runs;
+    }
+    if (a.run == NOISE_RUN || (uint64_t)a.count * a.runs_per_item <= 32ull * num_sms) return;
+    a.run = NOISE_RUN;
+  }
 }
 
 DeriveArgs derive_args(const lwe_ctx *c, const uint8_t *coins, const uint8_t *pkh,
@@ -407,7 +417,7 @@ int run_encrypt(lwe_ctx *c, const uint8_t *pk, const uint16_t *A, uint32_t count
     na.out[0] = noise_out(c->sp8, 8ull * n, 8 * n, 3, NOISE_I8);
   na.out[1] = noise_out(c->ep8, 8ull * n, 8 * n, 4, NOISE_I8);
   na.out[2] = noise_out(c->epp, 64, 64, 5, NOISE_I8);
-  noise_finish(na);
+  noise_finish(na, c->num_sms);
   LAUNCH(c, KID_NOISE, st, launch_noise(na, c->num_sms, st));
 
   if (tensor) {
@@ -492,7 +502,8 @@ void tree_hash(lwe_ctx *c, const uint8_t *msgs, uint64_t stride, uint32_t len, u
   ta.kprime = c->kp;
   ta.dig = c->tdig;
   ta.dig_words = c->tdig_words;
-  const uint32_t warp_max = warp_hash_max(c);
+  const uint32_t warp_max =
+      c->tree_warp_max < 0 ? tree_warp_max(c->num_sms, len) : (uint32_t)c->tree_warp_max;
   LAUNCH(c, count <= warp_max ? KID_TREE_WARP : KID_TREE, st,
          launch_tree(ta, c->num_sms, warp_max, st));
 }
@@ -977,6 +988,7 @@ int lwe_decaps_multi(lwe_ctx *c, const uint8_t *const *sk_ptrs, const uint16_t *
   DecryptArgs dca = decrypt_args(c, ct, nullptr, sk_ptrs);
   LAUNCH(c, KID_DECRYPT, st, launch_decrypt(dca, count, st));
   DeriveArgs da = derive_args(c, nullptr, nullptr, count);
+  da.flags = c->flags;
   da.pkh_ptrs = sk_ptrs;  // H(pk) is stored inside sk
   da.pkh_off = 8ull * n + 32;
   LAUNCH(c, KID_DERIVE, st, launch_derive(da, warp_hash_max(c), st));
@@ -1404,39 +1416,57 @@ struct lwe_pp_ctx {
   uint16_t *limbs = nullptr;   // [2][n][n] bf16 limbs of A
   uint32_t *partial = nullptr; // K-split running sums, [256][n] mod q
   bool tensor = false;         // LWE_PP_OPT_TENSOR (set when the GEMM supports n)
-  bool pdl = false;            // LWE_PP_OPT_PDL
+  bool pdl = true;             // LWE_PP_OPT_PDL
   // the key bound by lwe_pp_ctx_bind_key: its pk and A buffers, H(pk)
   // (bpkh), and whether `limbs` still holds the limbs of its A
   const uint8_t *bound_pk = nullptr;
   const uint32_t *bound_A = nullptr;
   uint8_t *bpkh = nullptr;
   bool limbs_bound = false;
+  // Decaps' H(c) runs beside the re-encryption
+  cudaStream_t side = nullptr;
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
 };
 
 namespace {
 
+void pp_ctx_free(lwe_pp_ctx *c) {
+  if (c->ev_fork) cudaEventDestroy(c->ev_fork);
+  if (c->ev_join) cudaEventDestroy(c->ev_join);
+  if (c->side) cudaStreamDestroy(c->side);
+  cudaFree(c->ws);
+  delete c;
+}
+
 void pp_tree(lwe_pp_ctx *c, const uint8_t *msgs, uint64_t stride, uint32_t len, uint32_t count,
-             int mode, uint8_t *out, uint64_t out_stride, cudaStream_t st) {
+             int mode, uint8_t *out, uint64_t out_stride, cudaStream_t st,
+             uint32_t tail_len = 0) {
   TreeArgs ta;
   memset(&ta, 0, sizeof ta);
   ta.msgs = msgs;
   ta.stride = stride;
   ta.len = len;
   ta.count = count;
+  ta.tail_len = tail_len;
   ta.mode = mode;
   ta.out = out;
   ta.out_stride = out_stride;
   ta.kprime = c->kp;
-  launch_tree(ta, c->num_sms, (uint32_t)c->num_sms, st);
+  launch_tree(ta, c->num_sms, tree_warp_max(c->num_sms, len), st);
 }
 
 // H(c) = Htree(Htree(u_0) || ... || Htree(u_255) || Htree(v)); with
 // TREE_ENC_KEY the last launch returns K = H(K' || H(c)) instead
 void pp_hash_ct(lwe_pp_ctx *c, const uint8_t *ct, int mode, uint8_t *out, cudaStream_t st) {
   const uint32_t row = 4 * c->p.n;
-  pp_tree(c, ct, row, row, PP_MBITS, TREE_DIGEST, c->digests, 32, st);
-  pp_tree(c, ct + (size_t)PP_MBITS * row, 4 * PP_MBITS, 4 * PP_MBITS, 1, TREE_DIGEST,
-          c->digests + 32 * PP_MBITS, 32, st);
+  if (4 * PP_MBITS <= row && PP_MBITS + 1 <= tree_warp_max(c->num_sms, row)) {
+    // v follows the rows: one launch for all 257
+    pp_tree(c, ct, row, row, PP_MBITS + 1, TREE_DIGEST, c->digests, 32, st, 4 * PP_MBITS);
+  } else {
+    pp_tree(c, ct, row, row, PP_MBITS, TREE_DIGEST, c->digests, 32, st);
+    pp_tree(c, ct + (size_t)PP_MBITS * row, 4 * PP_MBITS, 4 * PP_MBITS, 1, TREE_DIGEST,
+            c->digests + 32 * PP_MBITS, 32, st);
+  }
   pp_tree(c, c->digests, 32 * (PP_MBITS + 1), 32 * (PP_MBITS + 1), 1, mode, out, 32, st);
 }
 
