@@ -590,6 +590,7 @@ __global__ void __launch_bounds__(128) k_derive_warp(DeriveArgs a) {
   __syncthreads();
   pdl_wait();
   if (e >= a.count) return;  // the whole warp
+  if (a.flags && lane == 0) a.flags[e] = 0;
   const uint32_t nb = a.mu_bytes / 8;  // words of mu, 1..4
   uint32_t *mu = reinterpret_cast<uint32_t *>(a.mu + 32 * (size_t)e);
   const uint8_t *pkh = a.pkh_ptrs ? a.pkh_ptrs[e] + a.pkh_off : a.pkh + (size_t)e * a.pkh_stride;

@@ -1650,12 +1650,14 @@ int lwe_pp_ctx_create(const lwe_pp_params *p, int device, lwe_pp_ctx **out) {
     c->limbs = reinterpret_cast<uint16_t *>(c->ws + o_limbs);
     c->partial = reinterpret_cast<uint32_t *>(c->ws + o_partial);
   }
-  e = cudaMemset(c->ws, 0, off);
+  e = cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaMemset(c->ws, 0, off);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   cudaSetDevice(prev);
   if (e != cudaSuccess) {
-    cudaFree(c->ws);
-    delete c;
+    pp_ctx_free(c);
     return cuda_fail(e);
   }
   *out = c;
@@ -1670,7 +1672,6 @@ int lwe_pp_ctx_destroy(lwe_pp_ctx *c) {
   cudaDeviceSynchronize();
   pp_ctx_free(c);
   cudaSetDevice(prev);
-  delete c;
   return LWE_OK;
 }
 
@@ -1801,19 +1802,24 @@ int lwe_pp_decaps(lwe_pp_ctx *c, const uint8_t *sk, const uint32_t *A, const uin
   const uint32_t n = p.n;
   const uint8_t *z = sk + n, *pkh = sk + n + 32, *pk = sk + n + 64;
   PdlOn pdl(c->pdl);
-  CUDA_TRY(cudaMemsetAsync(c->flags, 0, 4, st));
+  CUDA_TRY(cudaEventRecord(c->ev_fork, st));
+  CUDA_TRY(cudaStreamWaitEvent(c->side, c->ev_fork, 0));
+  pp_hash_ct(c, ct, TREE_DIGEST, c->hc, c->side);
+  CUDA_TRY(cudaEventRecord(c->ev_join, c->side));
   CUDA_TRY(cudaMemsetAsync(c->mu, 0, 32, st));
   PpDecArgs dargs{reinterpret_cast<const uint32_t *>(ct),
                   reinterpret_cast<const uint32_t *>(ct) + (size_t)PP_MBITS * n,
                   reinterpret_cast<const int8_t *>(sk), reinterpret_cast<uint32_t *>(c->mu), n,
                   modq(p.q)};
   launch_pp_decrypt(dargs, st);  // m' into c->mu
-  launch_derive(pp_derive_args(c, nullptr, pkh), (uint32_t)c->num_sms, st);
+  DeriveArgs da = pp_derive_args(c, nullptr, pkh);
+  da.flags = c->flags;
+  launch_derive(da, (uint32_t)c->num_sms, st);
   pp_encrypt_noise(c, st);
   const int rc = pp_encrypt(c, reinterpret_cast<const uint32_t *>(pk + 16), A,
                             const_cast<uint8_t *>(ct), true, st);
+  CUDA_TRY(cudaStreamWaitEvent(st, c->ev_join, 0));
   if (rc != LWE_OK) return rc;
-  pp_hash_ct(c, ct, TREE_DIGEST, c->hc, st);
   FinalKeyArgs fa;
   memset(&fa, 0, sizeof fa);
   fa.kprime = c->kp;
