@@ -980,7 +980,7 @@ __global__ void __maxnreg__(112) k_tree_warp(TreeArgs a) {
   pdl_wait();
   const uint8_t *msg = a.msg_ptrs ? a.msg_ptrs[e] : a.msgs + (size_t)e * a.stride;
   const uint32_t dig0 = cluster_map(sdig, 0);
-  const uint32_t len = a.len;
+  const uint32_t len = a.tail_len && e == a.count - 1 ? a.tail_len : a.len;
   const uint32_t mc = (len + LWE_TREE_CHUNK - 1) / LWE_TREE_CHUNK;
   uint32_t s[5];
   for (uint32_t c0 = 3 * (q * nw + warp); c0 < mc; c0 += 3 * nq * nw) {
