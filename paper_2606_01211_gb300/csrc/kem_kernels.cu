@@ -120,41 +120,60 @@ LWE_DEV int tab_sample(const char *smem, uint32_t w16) {
   return *reinterpret_cast<const int8_t *>(smem + NOISE_TAB_OFF + w16);
 }
 
-LWE_DEV void noise_store(const char *smem, const NoiseOut &o, uint8_t *base, uint32_t b, uint4 v) {
+LWE_DEV void noise_store_i8(const int smp[8], uint8_t *base, uint32_t b, uint32_t nsamples) {
+  if (8 * b + 8 <= nsamples) {
+    const uint32_t lo = __byte_perm(__byte_perm(smp[0], smp[1], 0x0040),
+                                    __byte_perm(smp[2], smp[3], 0x0040), 0x5410);
+    const uint32_t hi = __byte_perm(__byte_perm(smp[4], smp[5], 0x0040),
+                                    __byte_perm(smp[6], smp[7], 0x0040), 0x5410);
+    *reinterpret_cast<uint2 *>(base + 8 * (size_t)b) = make_uint2(lo, hi);
+  } else {
+    for (int t = 0; t < 8; t++)
+      if (8 * b + t < nsamples) base[8 * (size_t)b + t] = (uint8_t)(int8_t)smp[t];
+  }
+}
+
+// small integers are exact in bf16
+LWE_DEV void noise_store_bf16(const int smp[8], uint8_t *base, uint32_t b, uint32_t nsamples) {
+  __nv_bfloat16 *bp = reinterpret_cast<__nv_bfloat16 *>(base);
+  if (8 * b + 8 <= nsamples) {
+    uint32_t pk[4];
+#pragma unroll
+    for (int t = 0; t < 4; t++) {
+      __nv_bfloat162 h2 = __floats2bfloat162_rn((float)smp[2 * t], (float)smp[2 * t + 1]);
+      pk[t] = *reinterpret_cast<uint32_t *>(&h2);
+    }
+    *reinterpret_cast<uint4 *>(bp + 8 * (size_t)b) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+  } else {
+    for (int t = 0; t < 8; t++)
+      if (8 * b + t < nsamples) bp[8 * (size_t)b + t] = __float2bfloat16_rn((float)smp[t]);
+  }
+}
+
+// PP: the paper profile's launches, with its two further formats
+template <bool PP>
+LWE_DEV void noise_store(const char *smem, const NoiseArgs &a, const NoiseOut &o, uint8_t *base,
+                         uint32_t b, uint4 v) {
   const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+  if (PP && o.fmt == NOISE_UNIFORM) {
+    int32_t *dst = reinterpret_cast<int32_t *>(base);
+    for (uint32_t t = 0; t < 8; t++) {
+      const uint32_t h = (w[t >> 1] >> (16 * (t & 1))) & 0xffffu;
+      if (8 * b + t < o.nsamples)
+        dst[8 * (size_t)b + t] = (int)(((2u * a.kunif + 1u) * h) >> 16) - (int)a.kunif;
+    }
+    return;
+  }
   int smp[8];
 #pragma unroll
   for (int t = 0; t < 4; t++) {
     smp[2 * t] = tab_sample(smem, w[t] & 0xffffu);
     smp[2 * t + 1] = tab_sample(smem, w[t] >> 16);
   }
-  const bool full = (8 * b + 8 <= o.nsamples);
-  if (o.fmt == NOISE_I8) {
-    if (full) {
-      const uint32_t lo = __byte_perm(__byte_perm(smp[0], smp[1], 0x0040),
-                                      __byte_perm(smp[2], smp[3], 0x0040), 0x5410);
-      const uint32_t hi = __byte_perm(__byte_perm(smp[4], smp[5], 0x0040),
-                                      __byte_perm(smp[6], smp[7], 0x0040), 0x5410);
-      *reinterpret_cast<uint2 *>(base + 8 * (size_t)b) = make_uint2(lo, hi);
-    } else {
-      for (int t = 0; t < 8; t++)
-        if (8 * b + t < o.nsamples) base[8 * (size_t)b + t] = (uint8_t)(int8_t)smp[t];
-    }
-  } else {  // bf16: small integers are exact
-    __nv_bfloat16 *bp = reinterpret_cast<__nv_bfloat16 *>(base);
-    if (full) {
-      uint32_t pk[4];
-#pragma unroll
-      for (int t = 0; t < 4; t++) {
-        __nv_bfloat162 h2 = __floats2bfloat162_rn((float)smp[2 * t], (float)smp[2 * t + 1]);
-        pk[t] = *reinterpret_cast<uint32_t *>(&h2);
-      }
-      *reinterpret_cast<uint4 *>(bp + 8 * (size_t)b) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-    } else {
-      for (int t = 0; t < 8; t++)
-        if (8 * b + t < o.nsamples) bp[8 * (size_t)b + t] = __float2bfloat16_rn((float)smp[t]);
-    }
-  }
+  if (o.fmt != NOISE_BF16) noise_store_i8(smp, base, b, o.nsamples);
+  if (o.fmt == NOISE_BF16 || (PP && o.fmt == NOISE_BOTH))
+    noise_store_bf16(smp, PP && o.fmt == NOISE_BOTH ? reinterpret_cast<uint8_t *>(o.base2) : base, b,
+                     o.nsamples);
 }
 
 // The runs of one warp: warp `gwarp` of `nwarps` takes runs gwarp,
@@ -195,6 +214,7 @@ LWE_DEV void noise_load_rk(const NoiseArgs &a, uint32_t e, uint32_t rk[44]) {
   }
 }
 
+template <bool PP>
 LWE_DEV void noise_runs(const NoiseArgs &a, const AesTab &tab, const char *smem, uint64_t gwarp,
                         uint64_t nwarps) {
   const uint32_t lane = threadIdx.x & 31;
@@ -233,18 +253,19 @@ LWE_DEV void noise_runs(const NoiseArgs &a, const AesTab &tab, const char *smem,
         for (uint32_t jj = 0; jj < NOISE_RUN / 32; jj += 2) {
           const uint4 va = aes_ctr_run_block(tab, rk, win, x0 + 32 * jj);
           const uint4 vb = aes_ctr_run_block(tab, rk, win, x0 + 32 * jj + 32);
-          noise_store(smem, o, base, b0 + 32 * jj, va);
-          noise_store(smem, o, base, b0 + 32 * jj + 32, vb);
+          noise_store<PP>(smem, a, o, base, b0 + 32 * jj, va);
+          noise_store<PP>(smem, a, o, base, b0 + 32 * jj + 32, vb);
         }
       } else {
 #pragma unroll 1
         for (uint32_t b = b0; b < min(nblk, first + a.run); b += 32)
-          noise_store(smem, o, base, b, aes_ctr_run_block(tab, rk, win, x0 + (b - b0)));
+          noise_store<PP>(smem, a, o, base, b, aes_ctr_run_block(tab, rk, win, x0 + (b - b0)));
       }
     }
   }
 }
 
+template <bool PP>
 __global__ void __launch_bounds__(512, 1) k_noise(NoiseArgs a) {
   extern __shared__ uint32_t sT[];
   pdl_trigger();
@@ -263,7 +284,7 @@ __global__ void __launch_bounds__(512, 1) k_noise(NoiseArgs a) {
   // large calls: a CTA's warps take consecutive runs (mostly one item's);
   // small ones: consecutive runs go to different SMs
   const uint64_t nw = blockDim.x >> 5, w = threadIdx.x >> 5;
-  noise_runs(a, tab, reinterpret_cast<const char *>(sT),
+  noise_runs<PP>(a, tab, reinterpret_cast<const char *>(sT),
              a.run == NOISE_RUN ? blockIdx.x * nw + w : w * gridDim.x + blockIdx.x, gridDim.x * nw);
 }
 
@@ -1356,8 +1377,10 @@ cudaError_t lwe_kernel_smem_setup() {
   cudaError_t e;
   e = cudaFuncSetAttribute(k_expand_A, cudaFuncAttributeMaxDynamicSharedMemorySize, AES_SMEM_BYTES);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_noise, cudaFuncAttributeMaxDynamicSharedMemorySize, NOISE_SMEM_BYTES);
-  if (e != cudaSuccess) return e;
+  for (auto k : {k_noise<false>, k_noise<true>}) {
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, NOISE_SMEM_BYTES);
+    if (e != cudaSuccess) return e;
+  }
   e = cudaFuncSetAttribute(k_noise_table, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            NOISE_SMEM_BYTES);
   if (e != cudaSuccess) return e;
@@ -1395,9 +1418,12 @@ void launch_noise_table(const NoiseArgs &a, int8_t *out, cudaStream_t st) {
   launch_k(k_noise_table, 1, 512, NOISE_SMEM_BYTES, st, a, out);
 }
 
-void launch_noise(const NoiseArgs &a, int num_sms, cudaStream_t st) {
+void launch_noise(const NoiseArgs &a, int num_sms, cudaStream_t st, bool pp) {
   const int g = grid_for((uint64_t)a.count * a.runs_per_item, a.run == NOISE_RUN ? 16 : 1, num_sms);
-  launch_k(k_noise, g, 512, NOISE_SMEM_BYTES, st, a);
+  if (pp)
+    launch_k(k_noise<true>, g, 512, NOISE_SMEM_BYTES, st, a);
+  else
+    launch_k(k_noise<false>, g, 512, NOISE_SMEM_BYTES, st, a);
 }
 
 void launch_mul_as(const MulAsArgs &a, uint32_t count, bool fused, int num_sms, cudaStream_t st) {

@@ -8,7 +8,9 @@
 // digests of their 1024-byte chunks (a fixed-shape two-level tree).
 #define LWE_TREE_CHUNK 1024
 
-enum { NOISE_I8 = 0, NOISE_BF16 = 1 };
+// NOISE_BOTH (int8 at base, bf16 at base2) and NOISE_UNIFORM (int32, centred
+// uniform on [-kunif, kunif]) only in the paper profile's launches
+enum { NOISE_I8 = 0, NOISE_BF16 = 1, NOISE_BOTH = 2, NOISE_UNIFORM = 3 };
 
 // Noise streams are cut into runs of consecutive counter blocks; one warp
 // generates one run, so one item's round keys serve a whole warp and the
@@ -24,8 +26,9 @@ struct NoiseOut {
   uint64_t item_stride;  // bytes
   uint32_t nsamples;     // samples per item, sample k from word k%8 of block k/8
   uint32_t domain;       // counter-block domain
-  uint32_t fmt;          // NOISE_I8 or NOISE_BF16
+  uint32_t fmt;          // NOISE_*
   uint32_t runs;         // ceil(ceil(nsamples / 8) / run)
+  void *base2;           // NOISE_BOTH, one item
 };
 
 struct NoiseArgs {
@@ -34,7 +37,7 @@ struct NoiseArgs {
   uint32_t nout;
   uint32_t runs_per_item;
   uint32_t run;          // blocks per run
-  uint32_t pad1, pad2;
+  uint32_t kunif, pad;
   NoiseOut out[3];
   uint32_t T[16];        // CDF table, entries >= clip set to 0x7FFF
   const uint4 *tab_img;  // the sampler table for T as k_noise_table writes it
@@ -168,7 +171,7 @@ cudaError_t lwe_upload_aes_table(const uint32_t T0[256]);
 cudaError_t lwe_kernel_smem_setup();
 void launch_expand_A(const uint8_t *seeds, uint32_t seed_stride, uint32_t count, uint32_t n,
                      uint32_t logq, uint16_t *A, uint64_t a_stride, int num_sms, cudaStream_t st);
-void launch_noise(const NoiseArgs &a, int num_sms, cudaStream_t st);
+void launch_noise(const NoiseArgs &a, int num_sms, cudaStream_t st, bool pp = false);
 void launch_noise_table(const NoiseArgs &a, int8_t *out, cudaStream_t st);
 void launch_mul_as(const MulAsArgs &a, uint32_t count, bool fused, int num_sms, cudaStream_t st);
 void launch_decrypt(const DecryptArgs &a, uint32_t count, cudaStream_t st);

@@ -309,7 +309,7 @@ NoiseArgs noise_args(const lwe_ctx *c, uint32_t count) {
 
 NoiseOut noise_out(void *base, uint64_t item_stride, uint32_t nsamples, uint32_t domain,
                    uint32_t fmt) {
-  return NoiseOut{base, item_stride, nsamples, domain, fmt, 0};
+  return NoiseOut{base, item_stride, nsamples, domain, fmt, 0, nullptr};
 }
 
 // Cuts the streams into runs: short ones while all of them fit two rounds of
@@ -1410,6 +1410,7 @@ struct lwe_pp_ctx {
   uint8_t *digests = nullptr;  // 257 x 32: the rows' and v's tree hashes
   uint32_t *rk = nullptr, *flags = nullptr;
   int8_t *e = nullptr, *Rt = nullptr, *E1t = nullptr;
+  int8_t *ntab = nullptr;      // the sampler table for T (64 KB), built at creation
   int32_t *e2 = nullptr;
   uint32_t *dev_err = nullptr;
   uint16_t *Rbf = nullptr;     // r^T as bf16 (GEMM operand)
@@ -1471,20 +1472,24 @@ void pp_hash_ct(lwe_pp_ctx *c, const uint8_t *ct, int mode, uint8_t *out, cudaSt
 }
 
 // Encrypt's noise from the round keys in c->rk: r, e1 (Gaussian, 256 x n)
-// and e2 (centred uniform, 256)
+// and e2 (centred uniform, 256).  The kernel of the matrix form's noise, whose
+// sampler is a table (17.8 us with up to 15 compares per sample, at n = 4096),
+// writes r as int8 and as the GEMM's bf16 at once (a conversion pass took 5.7).
 void pp_encrypt_noise(lwe_pp_ctx *c, cudaStream_t st) {
-  PpNoiseArgs na;
+  const uint32_t n = c->p.n;
+  NoiseArgs na;
   memset(&na, 0, sizeof na);
   na.rk = c->rk;
-  const uint32_t n = c->p.n;
-  na.o[0] = PpNoiseOut{c->Rt, PP_MBITS * n, PP_GAUSS, 3, 0};
-  na.o[1] = PpNoiseOut{c->E1t, PP_MBITS * n, PP_GAUSS, 4, 0};
-  na.o[2] = PpNoiseOut{c->e2, PP_MBITS, PP_UNIFORM, 5, 0};
-  na.nout = 3;
-  na.clip = c->p.clip;
+  na.count = 1;
+  na.tab_img = reinterpret_cast<const uint4 *>(c->ntab);
   na.kunif = c->p.k;
-  for (int i = 0; i < 16; i++) na.T[i] = c->T[i];
-  launch_pp_noise(na, c->num_sms, st);
+  na.nout = 3;
+  na.out[0] = noise_out(c->Rt, 0, PP_MBITS * n, 3, c->tensor ? NOISE_BOTH : NOISE_I8);
+  na.out[0].base2 = c->Rbf;
+  na.out[1] = noise_out(c->E1t, 0, PP_MBITS * n, 4, NOISE_I8);
+  na.out[2] = noise_out(c->e2, 0, PP_MBITS, 5, NOISE_UNIFORM);
+  noise_finish(na, c->num_sms);
+  launch_noise(na, c->num_sms, st, true);
 }
 
 // U^T and v of Encrypt from c's noise and message c->mu; cmp compares them
@@ -1500,7 +1505,6 @@ int pp_encrypt(lwe_pp_ctx *c, const uint32_t *t, const uint32_t *A, uint8_t *ct,
       launch_pp_limbs(A, n, c->p.q, c->limbs, st);
       c->limbs_bound = A == c->bound_A;
     }
-    launch_s_to_bf16(c->Rt, (uint64_t)PP_MBITS * n, c->Rbf, c->num_sms, st);
     GemmSaArgs ga;
     memset(&ga, 0, sizeof ga);
     ga.S = c->Rbf;
@@ -1616,6 +1620,7 @@ int lwe_pp_ctx_create(const lwe_pp_params *p, int device, lwe_pp_ctx **out) {
   const size_t o_hc = carve(32), o_dig = carve(32 * (PP_MBITS + 1)), o_rk = carve(176);
   const size_t o_flags = carve(16), o_e = carve(n), o_Rt = carve(PP_MBITS * n);
   const size_t o_E1t = carve(PP_MBITS * n), o_e2 = carve(4 * PP_MBITS), o_err = carve(16);
+  const size_t o_ntab = carve(65536);
   const bool tensor = lwe_gemm_supported((uint32_t)n, 16, p->clip);
   size_t o_Rbf = 0, o_limbs = 0, o_partial = 0;
   if (tensor) {
@@ -1640,6 +1645,7 @@ int lwe_pp_ctx_create(const lwe_pp_params *p, int device, lwe_pp_ctx **out) {
   c->rk = reinterpret_cast<uint32_t *>(c->ws + o_rk);
   c->flags = reinterpret_cast<uint32_t *>(c->ws + o_flags);
   c->e = reinterpret_cast<int8_t *>(c->ws + o_e);
+  c->ntab = reinterpret_cast<int8_t *>(c->ws + o_ntab);
   c->Rt = reinterpret_cast<int8_t *>(c->ws + o_Rt);
   c->E1t = reinterpret_cast<int8_t *>(c->ws + o_E1t);
   c->e2 = reinterpret_cast<int32_t *>(c->ws + o_e2);
@@ -1654,6 +1660,13 @@ int lwe_pp_ctx_create(const lwe_pp_params *p, int device, lwe_pp_ctx **out) {
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaMemset(c->ws, 0, off);
+  if (e == cudaSuccess) {
+    NoiseArgs na;
+    memset(&na, 0, sizeof na);
+    for (int i = 0; i < 16; i++) na.T[i] = c->T[i];
+    launch_noise_table(na, c->ntab, 0);
+    e = cudaGetLastError();
+  }
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   cudaSetDevice(prev);
   if (e != cudaSuccess) {
@@ -1734,7 +1747,6 @@ int lwe_pp_keygen(lwe_pp_ctx *c, const uint8_t *seed32, uint8_t *pk, uint8_t *sk
   na.o[1] = PpNoiseOut{c->e, n, PP_GAUSS, 2, 0};
   na.nout = 2;
   na.clip = p.clip;
-  na.kunif = p.k;
   for (int i = 0; i < 16; i++) na.T[i] = c->T[i];
   launch_pp_noise(na, c->num_sms, st);
   PpAsArgs aa{A, reinterpret_cast<const int8_t *>(sk), c->e, reinterpret_cast<uint32_t *>(pk + 16),

@@ -103,9 +103,9 @@ __global__ void __launch_bounds__(512, 1) k_pp_expand_A(const uint8_t *__restric
 }
 
 // ---------------------------------------------------------------------------
-// Noise streams (key schedule rk, one item): binomial eta = 3 from one byte
-// per sample, the CDF-table Gaussian from one 16-bit word, or the centred
-// uniform floor((2k + 1) w / 2^16) - k from one 16-bit word.
+// KeyGen's noise (key schedule rk, one item): binomial eta = 3 from one byte
+// per sample, the CDF-table Gaussian from one 16-bit word.  (Encrypt's 512 n
+// samples go through k_noise.)
 // ---------------------------------------------------------------------------
 LWE_DEV uint32_t pp_noise_blocks(const PpNoiseOut &o) {
   return o.kind == PP_BINOMIAL ? (o.count + 15) / 16 : (o.count + 7) / 8;
@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(512, 1) k_pp_noise(PpNoiseArgs a) {
   uint32_t rk[44];
 #pragma unroll
   for (int i = 0; i < 44; i++) rk[i] = a.rk[i];
-  uint32_t nb[3] = {0, 0, 0};
+  uint32_t nb[2] = {0, 0};
   uint64_t total = 0;
   for (uint32_t s = 0; s < a.nout; s++) {
     nb[s] = pp_noise_blocks(a.o[s]);
@@ -151,22 +151,12 @@ __global__ void __launch_bounds__(512, 1) k_pp_noise(PpNoiseArgs a) {
 #pragma unroll
       for (int t = 0; t < 8; t++) {
         const uint32_t h = (w[t >> 1] >> (16 * (t & 1))) & 0xffffu;
-        int e;
-        if (o.kind == PP_GAUSS) {
-          const uint32_t tt = h >> 1;
-          int mag = 0;
-          for (uint32_t i = 0; i < a.clip; i++) mag += tt > a.T[i] ? 1 : 0;
-          e = (h & 1u) ? -mag : mag;
-        } else {
-          e = (int)(((2u * a.kunif + 1u) * h) >> 16) - (int)a.kunif;
-        }
+        const uint32_t tt = h >> 1;
+        int mag = 0;
+        for (uint32_t i = 0; i < a.clip; i++) mag += tt > a.T[i] ? 1 : 0;
         const uint64_t idx = 8 * b + t;
-        if (idx < o.count) {
-          if (o.kind == PP_GAUSS)
-            reinterpret_cast<int8_t *>(o.out)[idx] = (int8_t)e;
-          else
-            reinterpret_cast<int32_t *>(o.out)[idx] = e;
-        }
+        if (idx < o.count)
+          reinterpret_cast<int8_t *>(o.out)[idx] = (int8_t)((h & 1u) ? -mag : mag);
       }
     }
   }

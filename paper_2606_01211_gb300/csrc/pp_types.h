@@ -11,7 +11,7 @@ struct ModQ {
   uint32_t q, m;
 };
 
-enum { PP_BINOMIAL = 0, PP_GAUSS = 1, PP_UNIFORM = 2 };
+enum { PP_BINOMIAL = 0, PP_GAUSS = 1 };
 
 struct PpNoiseOut {
   void *out;       // int8 (binomial, Gaussian) or int32 (uniform) samples
@@ -23,8 +23,8 @@ struct PpNoiseOut {
 
 struct PpNoiseArgs {
   const uint32_t *rk;  // 44 round-key words (device)
-  PpNoiseOut o[3];
-  uint32_t nout, clip, kunif, pad;
+  PpNoiseOut o[2];
+  uint32_t nout, clip;
   uint32_t T[16];      // CDF thresholds (clip used)
 };
 
