@@ -326,6 +326,18 @@ LWE_DEV uint32_t aes_last2(const AesTab &tab, uint32_t w0, uint32_t w1, uint32_t
   return ((tab.T<3, B0>(w0) & 0x000000ffu) ^ k) ^ (tab.T<1, B1>(w1) & 0x00ff0000u);
 }
 
+// The last round in full: the block's four words (rk: round key 10).
+LWE_DEV uint4 aes_last(const AesTab &tab, const uint32_t rk[4], const uint32_t s[4]) {
+  uint32_t o[4];
+#pragma unroll
+  for (int c = 0; c < 4; c++)
+    o[c] = ((tab.T<3, 0>(s[c]) & 0x000000ffu) | (tab.T<0, 1>(s[(c + 1) & 3]) & 0x0000ff00u) |
+            (tab.T<1, 2>(s[(c + 2) & 3]) & 0x00ff0000u) |
+            (tab.T<2, 3>(s[(c + 3) & 3]) & 0xff000000u)) ^
+           rk[c];
+  return make_uint4(o[0], o[1], o[2], o[3]);
+}
+
 // Load a 16-byte key from memory as four little-endian words.
 LWE_DEV void aes_load_key(const uint8_t *key, uint32_t k[4]) {
   if ((reinterpret_cast<uintptr_t>(key) & 15) == 0) {

@@ -1112,76 +1112,122 @@ LWE_DEV uint32_t limb_tile_at(uint32_t r, uint32_t c) {
 }
 
 // One instance per source of A: the stored one carries no AES state, so it
-// needs few registers and more CTAs per SM keep more loads in flight.
-template <bool FUSED>
-__global__ void __launch_bounds__(256) k_limbs(GemmLimbArgs a) {
+// needs few registers and more CTAs per SM keep more loads in flight.  The
+// regenerating one walks 64 x TC tiles with one CTA per SM, which fills the AES
+// tables once, TC / 64 blocks side by side per thread; a CTA per 64 x 64 tile,
+// as for the stored one, filled 128 KB for every 8 KB that it made.  TC = 64
+// where tiles of 128 would not fill the SMs, and NT = 256 threads where there
+// is one 64 x 64 tile per CTA, which leaves the other stream's kernels registers.
+// (Encaps and Decaps with the key not bound: 200 requests at n = 4096 832 ->
+// 678 us, 300 at 1344 269 -> 257.)
+template <bool FUSED, uint32_t TC, uint32_t NT>
+__global__ void __launch_bounds__(NT, !FUSED ? 6 : NT == 256 ? 3 : 1) k_limbs(GemmLimbArgs a) {
   extern __shared__ uint32_t sT[];
-  __shared__ __align__(16) uint16_t tile[64 * 64];
-  constexpr bool fused = FUSED;
-  const uint32_t n = a.n, ncols = n + (a.B ? 8u : 0u);
-  const uint32_t i0 = blockIdx.y * 64, c0 = blockIdx.x * 64;
+  constexpr uint32_t NH = 8 * TC / NT;  // 16-byte chunks per thread, FUSED
+  __shared__ __align__(16) uint16_t tile[64 * TC];
+  const uint32_t n = a.n, nch = n / 8, ncols = n + (a.B ? 8u : 0u), tid = threadIdx.x;
   const uint32_t mq = (1u << a.logq) - 1u, mm = mq | (mq << 16);
+  const uint32_t tiles_c = (ncols + TC - 1) / TC, tiles = tiles_c * ((n + 63) / 64);
+  auto at = [](uint32_t r, uint32_t c) { return (c >> 6) * 4096 + limb_tile_at(r, c & 63); };
+  // one or two tiles per CTA (TC = 64) do not pay for the index tables
+  constexpr bool USE_F = FUSED && TC == 128;
   AesTab tab;
-  uint32_t rk[44];
+  AesF F;
+  uint32_t rk[44];  // USE_F: round keys 3 .. 10 in the first 32
   pdl_trigger();
-  if (fused) {
+  if (FUSED) {
     aes_fill_smem(sT, g_aes_img);
     __syncthreads();
   }
   pdl_wait();
-  if (fused) {
+  if (FUSED && !USE_F) {
     tab = aes_tab(sT);
     uint32_t key[4];
     aes_load_key(a.seedA, key);
     aes_key_expand(tab, key, rk);
   }
-  for (uint32_t idx = threadIdx.x; idx < 512; idx += blockDim.x) {
-    const uint32_t r = idx >> 3, cq = idx & 7;
-    const uint32_t i = i0 + r, c = c0 + 8 * cq;
-    uint4 v = make_uint4(0, 0, 0, 0);
-    if (i < n) {
-      if (c + 8 <= n) {
-        if (fused) {
-          v = aes_ctr_block(tab, rk, 0, (uint64_t)i * (n / 8) + c / 8);
-          v.x &= mm;
-          v.y &= mm;
-          v.z &= mm;
-          v.w &= mm;
-        } else {
-          v = ld_nc_u4(a.A + (size_t)i * n + c);
-        }
-      } else if (a.B && c == n) {
-        v = ld_nc_u4(a.B + 16 * (size_t)i);
-      }
-    }
-    *reinterpret_cast<uint4 *>(&tile[limb_tile_at(r, 8 * cq)]) = v;
+  if (USE_F) {
+    uint4 *sF = reinterpret_cast<uint4 *>(reinterpret_cast<uint8_t *>(sT) + PRD_F_OFF);
+    uint32_t *srk = reinterpret_cast<uint32_t *>(reinterpret_cast<uint8_t *>(sT) + PRD_RK_OFF(1));
+    tab = aes_tab(sT);
+    if (prd_warp() == 0) prd_expand_key(tab, a.seedA, srk);
+    __syncthreads();
+    aes_f_fill(sF, tab, srk, 0, tid, NT);
+    __syncthreads();
+    prd_load_rk(srk, rk);
+    F = aes_f_open(sF, srk);
   }
-  __syncthreads();
-  for (uint32_t idx = threadIdx.x; idx < 512; idx += blockDim.x) {
-    const uint32_t cl = idx >> 3, ic = idx & 7;
-    const uint32_t c = c0 + cl, i = i0 + 8 * ic;
-    if (c >= ncols || i >= n) continue;
-    uint32_t lo[4], hi[4];
+  for (uint32_t tl = blockIdx.x; tl < tiles; tl += gridDim.x) {
+    const uint32_t c0 = (tl % tiles_c) * TC, i0 = tl / tiles_c * 64;
+    if (FUSED) {
+      constexpr uint32_t RP = 64 / NH;  // rows per pass of the threads
+      const uint32_t cq = tid % (TC / 8), r = tid / (TC / 8), c = c0 + 8 * cq;
+      uint4 v[NH];
+      if (c < n) {  // rows beyond n are counters whose blocks nothing reads
+        uint32_t s[NH][4];
+        if (USE_F) {
 #pragma unroll
-    for (int t = 0; t < 8; t += 2) {
-      float fl[2], fh[2];
+          for (uint32_t h = 0; h < NH; h++)
+            aes_f_start(F, tab, 0, (i0 + r + RP * h) * nch + c / 8, s[h]);
+          aes_rounds_3_9<NH>(tab, rk, s);
+        }
 #pragma unroll
-      for (int u = 0; u < 2; u++) {
-        const int x = tile[limb_tile_at(8 * ic + t + u, cl)];
-        const int l = (int)(int8_t)(uint8_t)(x & 0xff);
-        const int h = (int)(int8_t)(uint8_t)(((x - l) >> 8) & 0xff);
-        fl[u] = (float)l;
-        fh[u] = (float)h;
+        for (uint32_t h = 0; h < NH; h++) {
+          v[h] = USE_F ? aes_last(tab, rk + 28, s[h])
+                       : aes_ctr_block(tab, rk, 0, (uint64_t)(i0 + r + RP * h) * nch + c / 8);
+          v[h] = make_uint4(v[h].x & mm, v[h].y & mm, v[h].z & mm, v[h].w & mm);
+        }
+      } else {
+#pragma unroll
+        for (uint32_t h = 0; h < NH; h++)
+          v[h] = a.B && c == n && i0 + r + RP * h < n ? ld_nc_u4(a.B + 16 * (size_t)(i0 + r + RP * h))
+                                                      : make_uint4(0, 0, 0, 0);
       }
-      __nv_bfloat162 bl = __floats2bfloat162_rn(fl[0], fl[1]);
-      __nv_bfloat162 bh = __floats2bfloat162_rn(fh[0], fh[1]);
-      lo[t / 2] = *reinterpret_cast<uint32_t *>(&bl);
-      hi[t / 2] = *reinterpret_cast<uint32_t *>(&bh);
+#pragma unroll
+      for (uint32_t h = 0; h < NH; h++)
+        *reinterpret_cast<uint4 *>(&tile[at(r + RP * h, 8 * cq)]) = v[h];
+    } else {
+      for (uint32_t idx = tid; idx < 512; idx += NT) {
+        const uint32_t r = idx >> 3, cq = idx & 7;
+        const uint32_t i = i0 + r, c = c0 + 8 * cq;
+        uint4 v = make_uint4(0, 0, 0, 0);
+        if (i < n) {
+          if (c + 8 <= n)
+            v = ld_nc_u4(a.A + (size_t)i * n + c);
+          else if (a.B && c == n)
+            v = ld_nc_u4(a.B + 16 * (size_t)i);
+        }
+        *reinterpret_cast<uint4 *>(&tile[at(r, 8 * cq)]) = v;
+      }
     }
-    uint16_t *L = a.limbs;
-    *reinterpret_cast<uint4 *>(L + (size_t)c * n + i) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-    *reinterpret_cast<uint4 *>(L + ((size_t)ncols + c) * n + i) =
-        make_uint4(hi[0], hi[1], hi[2], hi[3]);
+    __syncthreads();
+    for (uint32_t idx = tid; idx < 8 * TC; idx += NT) {
+      const uint32_t cl = idx >> 3, ic = idx & 7;
+      const uint32_t c = c0 + cl, i = i0 + 8 * ic;
+      if (c >= ncols || i >= n) continue;
+      uint32_t lo[4], hi[4];
+#pragma unroll
+      for (int t = 0; t < 8; t += 2) {
+        float fl[2], fh[2];
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+          const int x = tile[at(8 * ic + t + u, cl)];
+          const int l = (int)(int8_t)(uint8_t)(x & 0xff);
+          const int h = (int)(int8_t)(uint8_t)(((x - l) >> 8) & 0xff);
+          fl[u] = (float)l;
+          fh[u] = (float)h;
+        }
+        __nv_bfloat162 bl = __floats2bfloat162_rn(fl[0], fl[1]);
+        __nv_bfloat162 bh = __floats2bfloat162_rn(fh[0], fh[1]);
+        lo[t / 2] = *reinterpret_cast<uint32_t *>(&bl);
+        hi[t / 2] = *reinterpret_cast<uint32_t *>(&bh);
+      }
+      uint16_t *L = a.limbs;
+      *reinterpret_cast<uint4 *>(L + (size_t)c * n + i) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+      *reinterpret_cast<uint4 *>(L + ((size_t)ncols + c) * n + i) =
+          make_uint4(hi[0], hi[1], hi[2], hi[3]);
+    }
+    if (FUSED) __syncthreads();  // the tile is read before the next one is written
   }
 }
 
@@ -1402,7 +1448,10 @@ cudaError_t lwe_kernel_smem_setup() {
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_pp_noise, cudaFuncAttributeMaxDynamicSharedMemorySize, AES_SMEM_BYTES);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_limbs<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, AES_SMEM_BYTES);
+  for (auto k : {k_limbs<true, 64, 256>, k_limbs<true, 64, 512>, k_limbs<true, 128, 512>}) {
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, PRD_SMEM);
+    if (e != cudaSuccess) return e;
+  }
   return e;
 }
 
@@ -1637,13 +1686,17 @@ void launch_final_key(const FinalKeyArgs &a, uint32_t warp_max, cudaStream_t st)
 }
 
 void launch_gemm_limbs(const GemmLimbArgs &a, int num_sms, cudaStream_t st) {
-  (void)num_sms;
-  const uint32_t ncols = a.n + (a.B ? 8u : 0u);
-  dim3 grid((ncols + 63) / 64, (a.n + 63) / 64);
+  const uint32_t ncols = a.n + (a.B ? 8u : 0u), rows = (a.n + 63) / 64;
+  const uint32_t sms = (uint32_t)std::max(num_sms, 1), t64 = (ncols + 63) / 64 * rows;
+  const uint32_t t128 = (ncols + 127) / 128 * rows;
   if (a.A)
-    launch_k(k_limbs<false>, grid, 256, 0, st, a);
+    launch_k(k_limbs<false, 64, 256>, t64, 256, 0, st, a);
+  else if (t64 <= sms)
+    launch_k(k_limbs<true, 64, 256>, t64, 256, AES_SMEM_BYTES, st, a);
+  else if (t128 < sms)
+    launch_k(k_limbs<true, 64, 512>, sms, 512, AES_SMEM_BYTES, st, a);
   else
-    launch_k(k_limbs<true>, grid, 256, AES_SMEM_BYTES, st, a);
+    launch_k(k_limbs<true, 128, 512>, std::min(t128, sms), 512, PRD_SMEM, st, a);
 }
 
 void launch_s_to_bf16(const int8_t *S, uint64_t count, uint16_t *out, int num_sms, cudaStream_t st) {
