@@ -1608,6 +1608,13 @@ void launch_tree(TreeArgs &a, int num_sms, uint32_t warp_max, cudaStream_t st) {
     launch_k_cluster(k_tree_warp, a.count * q, 32 * w, (size_t)a.m * 32, st, q, a);
     return;
   }
+  auto two_launches = [&] {
+    // small leaf CTAs when the batch fills the SMs only a few warps deep
+    const uint64_t leaves = (uint64_t)a.count * a.m;
+    const uint32_t lt = leaves >= (uint64_t)sms * 1024 ? 256u : 64u;
+    launch_k(k_tree_leaves, (uint32_t)((leaves + lt - 1) / lt), lt, 0, st, a);
+    launch_k(k_tree_roots, (a.count + 5) / 6, 64, 0, st, a);
+  };
   if (a.m > 32 && dig_fits) {
     // long messages: every leaf on its own thread, then one warp per root,
     // once k_tree (below: one thread per message runs its root) would have
@@ -1618,11 +1625,7 @@ void launch_tree(TreeArgs &a, int num_sms, uint32_t warp_max, cudaStream_t st) {
     const uint32_t cap = std::max<uint32_t>(
         1u, std::min<uint32_t>(TREE_MAX_THREADS / t, (48u * 1024u) / (8u * (4 * a.m + 1))));
     if (a.m > 128 || a.count > 2 * sms * cap) {
-      // small leaf CTAs when the batch fills the SMs only a few warps deep
-      const uint64_t leaves = (uint64_t)a.count * a.m;
-      const uint32_t lt = leaves >= (uint64_t)sms * 1024 ? 256u : 64u;
-      launch_k(k_tree_leaves, (uint32_t)((leaves + lt - 1) / lt), lt, 0, st, a);
-      launch_k(k_tree_roots, (a.count + 5) / 6, 64, 0, st, a);
+      two_launches();
       return;
     }
   }
@@ -1662,6 +1665,12 @@ void launch_tree(TreeArgs &a, int num_sms, uint32_t warp_max, cudaStream_t st) {
       launch_k(k_tree_dense, (a.count + ipc - 1) / ipc, 512, smem_d, st, a);
       return;
     }
+  }
+  if (a.m >= 2 && dig_fits) {
+    // more leaves than 13 warps per SM (or than 32 messages): Encaps of 4096
+    // requests at n = 1344, 22 leaves each, 826 us with k_tree, 704 so
+    two_launches();
+    return;
   }
   uint32_t t = 1;
   while (t < a.m && t < 256) t <<= 1;
