@@ -869,15 +869,44 @@ __global__ void __maxnreg__(96) k_tree_bal(TreeArgs a) {
   }
 }
 
+// The end of a tree hash (s: the final state of each group's root, message e
+// of the group if `in`): digest mode stores H into out (and out2); Encaps mode
+// derives K = H(K' || H(c)) (Alg. 4), one 64-byte block.
+LWE_DEV void tree_tri_out(const TreeArgs &a, uint32_t e, bool in, const KeccakTri &km,
+                          uint32_t lane, uint32_t s[5]) {
+  uint32_t v = tri_digest_word(km, s);
+  const bool st = in && lane < 30 && km.r < 8;
+  if (a.mode == TREE_DIGEST) {
+    if (st) st_le32(a.out + (size_t)e * a.out_stride + 4 * km.r, v);
+    if (st && a.out2) st_le32(a.out2 + (size_t)e * a.out2_stride + 4 * km.r, v);
+    return;
+  }
+  uint64_t hc[4];
+#pragma unroll
+  for (uint32_t i = 0; i < 4; i++)
+    hc[i] = (uint64_t)tri_shfl(v, 10 * km.grp + 2 * i) |
+            ((uint64_t)tri_shfl(v, 10 * km.grp + 2 * i + 1) << 32);
+  const uint64_t *kp = reinterpret_cast<const uint64_t *>(a.kprime + 32 * (size_t)(in ? e : 0));
+  tri_one_block(km, s, [&](uint32_t w) -> uint64_t {
+    uint64_t x = sha3_pad_word(w, 8);
+    if (w < 4) x ^= kp[w];
+#pragma unroll
+    for (uint32_t i = 0; i < 4; i++) x ^= w == 4 + i ? hc[i] : 0ull;
+    return x;
+  });
+  v = tri_digest_word(km, s);
+  if (st) st_le32(a.out + 32 * (size_t)e + 4 * km.r, v);
+}
+
 // Tree hash of batches whose full-length leaves fill at most 12 warps per
 // CTA (e.g. 4096 ciphertexts of n = 640: 27 per SM, 270 leaves): the leaves
 // are packed densely, leaf k on warp k / 32 of warps 0-11, so consecutive
 // warps fall on consecutive SM sub-partitions and every SMSP holds
 // floor or ceil of WL / 4 leaf warps (k_tree instead gives each message a
 // power-of-two group of threads, which leaves lanes idle).  The short last
-// chunks and then the roots (and Encaps' key) run on one warp of the SMSP
-// with the fewest leaf warps, `rw`.  One named barrier: the twelve leaf
-// warps (whether or not they hold leaves) -> the root warp (416 threads).
+// chunks run on one warp of the SMSP with the fewest leaf warps, `rw`; then,
+// behind one named barrier (the twelve leaf warps, whether or not they hold
+// leaves, and rw: 416 threads), the roots.
 __global__ void __maxnreg__(96) k_tree_dense(TreeArgs a) {
   extern __shared__ uint64_t sm[];
   pdl_trigger();
@@ -911,70 +940,30 @@ __global__ void __maxnreg__(96) k_tree_dense(TreeArgs a) {
         sha3_absorb_global(msg_of(li) + (size_t)c * LWE_TREE_CHUNK, LWE_TREE_CHUNK, 0, fullp, s);
       put_digest(li, c, s);
     }
-    __syncwarp();
-    bar_arrive(1, 416);
+  } else if (warp != a.rw) {
     return;
-  }
-  if (warp != a.rw) return;
-  const uint32_t li = lane;
-  const bool mine = li < nmsg;
-  if (mine && ML < a.m) {
-    const uint32_t c = a.m - 1, off = c * LWE_TREE_CHUNK, len = a.len - off;
-    sha3_init(s);
-    if (LWE_BOUNDS(off < a.len && len <= LWE_TREE_CHUNK, 113))
-      sha3_absorb_global(msg_of(li) + off, len, 0, len / SHA3_RATE + 1, s);
-    put_digest(li, c, s);
+  } else {
+    const uint32_t li = lane;
+    if (li < nmsg && ML < a.m) {
+      const uint32_t c = a.m - 1, off = c * LWE_TREE_CHUNK, len = a.len - off;
+      sha3_init(s);
+      if (LWE_BOUNDS(off < a.len && len <= LWE_TREE_CHUNK, 113))
+        sha3_absorb_global(msg_of(li) + off, len, 0, len / SHA3_RATE + 1, s);
+      put_digest(li, c, s);
+    }
   }
   __syncwarp();
   bar_sync(1, 416);
-  if (!mine) return;
-  const uint32_t rlen = 32 * a.m;
-  sha3_init(s);
-  sha3_absorb_mem(reinterpret_cast<const uint8_t *>(sdig + (size_t)li * words), rlen, 0,
-                  rlen / SHA3_RATE + 1, s);
-  const uint32_t e = e0 + li;
-  if (a.mode == TREE_DIGEST) {
-    sha3_digest(s, a.out + (size_t)e * a.out_stride);
-    if (a.out2) sha3_digest(s, a.out2 + (size_t)e * a.out2_stride);
-  } else {
-    // Encaps (Alg. 4): K = H(K' || H(c))
-    uint64_t lanes[SHA3_RATE / 8];
-    lanes_zero(lanes);
-    const uint64_t *kp = reinterpret_cast<const uint64_t *>(a.kprime + 32 * (size_t)e);
-    for (int i = 0; i < 4; i++) lanes[i] = kp[i];
-    for (int i = 0; i < 4; i++) lanes[4 + i] = s[i];
-    sha3_256_lanes(lanes, 64, s);
-    sha3_digest(s, a.out + 32 * (size_t)e);
-  }
-}
-
-// The end of a tree hash (s: the final state of each group's root, message e
-// of the group if `in`): digest mode stores H into out (and out2); Encaps mode
-// derives K = H(K' || H(c)) (Alg. 4), one 64-byte block.
-LWE_DEV void tree_tri_out(const TreeArgs &a, uint32_t e, bool in, const KeccakTri &km,
-                          uint32_t lane, uint32_t s[5]) {
-  uint32_t v = tri_digest_word(km, s);
-  const bool st = in && lane < 30 && km.r < 8;
-  if (a.mode == TREE_DIGEST) {
-    if (st) st_le32(a.out + (size_t)e * a.out_stride + 4 * km.r, v);
-    if (st && a.out2) st_le32(a.out2 + (size_t)e * a.out2_stride + 4 * km.r, v);
-    return;
-  }
-  uint64_t hc[4];
-#pragma unroll
-  for (uint32_t i = 0; i < 4; i++)
-    hc[i] = (uint64_t)tri_shfl(v, 10 * km.grp + 2 * i) |
-            ((uint64_t)tri_shfl(v, 10 * km.grp + 2 * i + 1) << 32);
-  const uint64_t *kp = reinterpret_cast<const uint64_t *>(a.kprime + 32 * (size_t)(in ? e : 0));
-  tri_one_block(km, s, [&](uint32_t w) -> uint64_t {
-    uint64_t x = sha3_pad_word(w, 8);
-    if (w < 4) x ^= kp[w];
-#pragma unroll
-    for (uint32_t i = 0; i < 4; i++) x ^= w == 4 + i ? hc[i] : 0ull;
-    return x;
-  });
-  v = tri_digest_word(km, s);
-  if (st) st_le32(a.out + 32 * (size_t)e + 4 * km.r, v);
+  // the roots (and Encaps' keys), three per warp: chains of 4-5 permutations
+  // at ~2.3 us each where one warp of one root per thread took 4.7
+  if (3 * warp >= nmsg) return;
+  const KeccakTri km = keccak_tri(lane);
+  const uint32_t li = 3 * warp + km.grp;
+  const bool in = li < nmsg;
+  uint32_t st[5];
+  sha3_256_tri<false>(km, reinterpret_cast<const uint8_t *>(sdig + (size_t)(in ? li : 0) * words),
+                      in ? 32 * a.m : 0u, st);
+  tree_tri_out(a, e0 + li, in, km, lane, st);
 }
 
 // Tree hash with three Keccak states per warp (keccak_warp.cuh), for launches
