@@ -230,12 +230,14 @@ LWE_DEV uint64_t tri_msg_word(const uint8_t *msg, uint32_t len, uint32_t blk, ui
   return v;
 }
 
-// SHA3-256 of each group's message (msg, len are the group's; a group without
-// one passes len 0 and ignores its digest).  The warp runs as many
-// permutations as its longest message; a group that is done keeps its state.
-// The next block's words are fetched before a permutation.
+// Absorbs blocks k0 .. of each group's message, to its end (msg, len are the
+// group's, k0 the warp's; a group without a message passes len 0 and ignores
+// its digest).  The warp runs as many permutations as its longest message
+// needs; a group that is done keeps its state.  The next block's words are
+// fetched before a permutation.
 template <bool GLB>
-LWE_DEV void sha3_256_tri(const KeccakTri &m, const uint8_t *msg, uint32_t len, uint32_t s[5]) {
+LWE_DEV void sha3_absorb_tri(const KeccakTri &m, const uint8_t *msg, uint32_t len, uint32_t k0,
+                             uint32_t s[5]) {
   const uint32_t full = len / SHA3_RATE, nblk = full + 1;
   const uint32_t most = __reduce_max_sync(0xffffffffu, nblk);
   uint32_t lane[5];
@@ -253,11 +255,10 @@ LWE_DEV void sha3_256_tri(const KeccakTri &m, const uint8_t *msg, uint32_t len, 
   };
 #pragma unroll
   for (uint32_t i = 0; i < 5; i++) {
-    s[i] = 0;
     lane[i] = tri_lane(m, i);
   }
-  fetch(0);
-  for (uint32_t k = 0; k < most; k++) {
+  fetch(k0);
+  for (uint32_t k = k0; k < most; k++) {
     uint32_t v[5];
 #pragma unroll
     for (uint32_t i = 0; i < 5; i++) v[i] = s[i] ^ tri_half(w[i], m.h);
@@ -266,4 +267,12 @@ LWE_DEV void sha3_256_tri(const KeccakTri &m, const uint8_t *msg, uint32_t len, 
 #pragma unroll
     for (uint32_t i = 0; i < 5; i++) s[i] = k < nblk ? v[i] : s[i];
   }
+}
+
+// SHA3-256 of each group's message.
+template <bool GLB>
+LWE_DEV void sha3_256_tri(const KeccakTri &m, const uint8_t *msg, uint32_t len, uint32_t s[5]) {
+#pragma unroll
+  for (uint32_t i = 0; i < 5; i++) s[i] = 0;
+  sha3_absorb_tri<GLB>(m, msg, len, 0, s);
 }

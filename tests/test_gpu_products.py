@@ -55,3 +55,19 @@ def test_many_regenerated_items_match_oracle(n, count):
         assert np.array_equal(pk_h[i], pk_o), i
         assert np.array_equal(sk_h[i], sk_o), i
     ctx.close()
+
+
+@pytest.mark.parametrize("n", [512, 528, 4112])
+def test_products_exact_at_the_largest_sums(n):
+    """Every byte of A 255 and S = -128: the accumulators reach their bound,
+    512 terms of 255 x 128 below 2^24, and are emptied in time beyond it."""
+    A = np.full((n, n), 0xFFFF, dtype=np.uint16)
+    S = np.full((8, n), -128, dtype=np.int8)
+    S[1::2] = 127
+    A_d = dev(A.view(np.int16))
+    out = torch.empty((n, 8), dtype=torch.int16, device="cuda")
+    lwe.matmul_modq(lwe.SIDE_AS, dev(S), out, n, 16, A=A_d)
+    assert np.array_equal(as_u16(out), O.mul_AS(A, S, None, 16))
+    out2 = torch.empty((8, n), dtype=torch.int16, device="cuda")
+    lwe.matmul_modq(lwe.SIDE_SA, dev(S), out2, n, 16, A=A_d)
+    assert np.array_equal(as_u16(out2), O.mul_SA(S, A, None, 16))

@@ -32,3 +32,28 @@ def test_key_hash_matches_hashlib(n, count):
         got = sk_h[i, 8 * n + 32:8 * n + 64].tobytes()
         assert got == _tree(pk_h[i].tobytes()), i
     ctx.close()
+
+
+@pytest.mark.parametrize("n,count", [(400, 10700), (1344, 2900), (1344, 2750), (976, 3990),
+                                     (640, 1501)])
+def test_batch_schedules_agree_with_it(n, count):
+    """Encaps' keys from the batched tree schedules (two launches for more than
+    32 messages or 13 leaf warps per SM; the balanced and the dense one with
+    their roots three per warp) equal those of one message per CTA; ragged
+    last CTAs."""
+    torch.cuda.set_device(0)
+    p, _ = params("P640", n=n, logq=16)
+    ctx = lwe.Ctx(p, max_batch=count)
+    pk, sk = ctx.empty_pk(1), ctx.empty_sk(1)
+    ctx.keygen(dev(master_seeds(1, seed=n)), pk, sk)
+    coins = dev(np.random.default_rng(n).integers(0, 256, (count, 32), dtype=np.uint8))
+    ct = ctx.empty_ct(count)
+    keys = []
+    for warp_max in (-1, count):
+        K = torch.empty((count, 32), dtype=torch.uint8, device="cuda")
+        ctx.set_option(lwe.OPT_WARP_HASH_MAX, warp_max)
+        ctx.encaps(pk, coins, ct, K)
+        keys.append(host(K))
+    assert np.array_equal(keys[0], keys[1])
+    assert ctx.device_error() == 0
+    ctx.close()
