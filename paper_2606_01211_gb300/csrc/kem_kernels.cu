@@ -59,7 +59,8 @@ __global__ void __launch_bounds__(512, 1) k_expand_A(const uint8_t *__restrict__
   // passed to the warp by shuffles as in noise_runs
   const uint32_t lane = threadIdx.x & 31;
   const uint64_t nruns = (nblk + 127) / 128, nw = (uint64_t)gridDim.x * (blockDim.x >> 5);
-  const uint64_t gw = (uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  // (warp-major: the runs of the last, partial round go to all SMs alike)
+  const uint64_t gw = (uint64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
   for (uint64_t g = 0; gw + nw * g < nruns; g += 32) {
     AesCtrRun mine{};
     if (gw + nw * (g + lane) < nruns) mine = aes_ctr_run(tab, rk, 0, (gw + nw * (g + lane)) * 128);

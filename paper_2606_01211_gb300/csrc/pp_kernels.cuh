@@ -82,8 +82,8 @@ __global__ void __launch_bounds__(512, 1) k_pp_expand_A(const uint8_t *__restric
   uint4 *out = reinterpret_cast<uint4 *>(A);
   const uint32_t lane = threadIdx.x & 31;
   const uint64_t nruns = (nblk + 127) / 128, nw = (uint64_t)gridDim.x * (blockDim.x >> 5);
-  for (uint64_t run = (uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); run < nruns;
-       run += nw) {
+  // (warp-major: the runs of the last, partial round go to all SMs alike)
+  for (uint64_t run = (uint64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; run < nruns; run += nw) {
     const uint64_t first = run * 128;
     const AesCtrRun win = aes_ctr_run(tab, rk, PP_A_DOMAIN, first);
     const uint32_t x0 = (uint32_t)(first & 255u) + lane;
