@@ -324,8 +324,8 @@ LIMITER = {
     "k_noise": "shared-memory pipe: AES round-table lookups plus the sampler's table",
     "k_tree": "integer ALU pipe: Keccak-f XORs, rotations and chi; the balanced schedule "
               "(k_tree_bal) hands SM sub-partition 0's leaves to helper warps after 6 of 8 "
-              "permutations and absorbs the roots in two stages: about 33 warp-permutations "
-              "on the critical path against 29 of work",
+              "permutations; the roots' first blocks are absorbed meanwhile, their last ones "
+              "three per warp once the leaves are done",
     "k_gemm_tc": "tensor pipe (bf16 tcgen05, CTA pairs)",
 }
 
@@ -355,18 +355,20 @@ def algorithmic(p, count):
 CSRC = os.path.join(ROOT, "paper_2606_01211_gb300", "csrc")
 TRAFFIC = {
     # kernel: (bytes per step, launches per step, [(file, function or None)], fingerprint, profile)
-    "k_tree": (129.280000e6, 2,
+    "k_tree": (129.379584e6, 2,
                [("kem_kernels.cu", "k_tree_bal"), ("kem_kernels.cu", "launch_tree"),
-                ("keccak.cuh", None)],
-               "61a10e1e45bb906c", "profiles/k_tree_p976.md"),
-    "k_gemm_tc": (295.779584e6, 2, [("gemm_tc.cu", None)], "10f4eabbb5ca2195",
+                ("kem_kernels.cu", "tree_tri_out"), ("keccak.cuh", None),
+                ("keccak_warp.cuh", None)],
+               "761cb1539b8e7e03", "profiles/k_tree_p976.md"),
+    "k_gemm_tc": (295.791104e6, 2, [("gemm_tc.cu", None)], "a11460dc8c0e227f",
                   "profiles/k_gemm_sa2_p976.md"),
-    "k_noise": (69.913344e6, 2,
+    "k_noise": (69.633280e6, 2,
                 [("kem_kernels.cu", "k_noise"), ("kem_kernels.cu", "noise_runs"),
-                 ("kem_kernels.cu", "noise_store"),
+                 ("kem_kernels.cu", "noise_store"), ("kem_kernels.cu", "noise_store_i8"),
+                 ("kem_kernels.cu", "noise_store_bf16"),
                  ("kem_kernels.cu", "noise_fill_table"), ("kem_kernels.cu", "launch_noise"),
                  ("aes.cuh", None)],
-                "8c69346ce7bf41c6", "profiles/k_noise_p976.md"),
+                "b6198af6ae45c6f4", "profiles/k_noise_p976.md"),
 }
 
 

@@ -380,8 +380,8 @@ int lwe_bounds_violations(uint64_t *count, uint32_t *first_site);
  *     permutation of k_tree).  Work: ctas * 256 * iters permutations.
  *   LWE_PROBE_AES: `ctas` CTAs of 512 threads with the AES round tables in
  *     shared memory; each thread encrypts `iters` (even) counter blocks, two
- *     at a time, every round in full (the generator of the kernels whose
- *     blocks do not run along one counter window, e.g. S' A with A
+ *     at a time, every round in full (the first rounds neither windowed, as
+ *     LWE_PROBE_AES_RUN, nor from index tables, as the products with A
  *     regenerated).  Work: ctas * 512 * iters blocks.
  *   LWE_PROBE_AES_RUN: as LWE_PROBE_AES with the blocks of a warp taken
  *     four per lane from one 128-block run of counter indices, whose first

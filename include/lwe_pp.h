@@ -75,8 +75,8 @@ int lwe_pp_ctx_destroy(lwe_pp_ctx *ctx);
  * epilogue); 0 on the CUDA cores (int32 multiply-adds).  LWE_PP_OPT_PDL: 1
  * (default) launches the kernels of a call with programmatic stream
  * serialisation (as LWE_OPT_PDL of lwe.h); 0: plain launches (a cycle of
- * KeyGen, Encaps and Decaps at n = 512 / 4096 / 8192: 273 / 531 / 1044 us with,
- * 305 / 537 / 1059 us without). */
+ * KeyGen, Encaps and Decaps at n = 2048 / 4096 / 8192 / 16384 / 32768: 290 /
+ * 454 / 996 / 2683 / 9465 us with, 316 / 490 / 1008 / 2750 / 9492 without). */
 enum { LWE_PP_OPT_TENSOR = 0, LWE_PP_OPT_PDL = 1 };
 int lwe_pp_ctx_set_option(lwe_pp_ctx *ctx, int option, int64_t value);
 

@@ -313,7 +313,7 @@ NoiseOut noise_out(void *base, uint64_t item_stride, uint32_t nsamples, uint32_t
 }
 
 // Cuts the streams into runs: short ones while all of them fit two rounds of
-// the SMs' 16 warps (one request: 12 -> 4.5 us at n = 1344), else NOISE_RUN.
+// the SMs' 16 warps (a request at n = 640 181 -> 174 us, at 1344 116 -> 111), else NOISE_RUN.
 void noise_finish(NoiseArgs &a, int num_sms) {
   a.run = NOISE_RUN_SMALL;
   for (;;) {
