@@ -134,13 +134,17 @@ enum {
   LWE_OPT_PATH = 0,          /* one of LWE_PATH_*                             */
   LWE_OPT_TENSOR_MIN = 1,    /* AUTO threshold (items per call), default 64   */
   LWE_OPT_TIMING = 2,        /* 1: time every launch with CUDA events          */
-  LWE_OPT_GEMM_BN = 3,       /* single-CTA GEMM column tile: 64 or 128 (def.) */
+  LWE_OPT_GEMM_BN = 3,       /* column tile with LWE_OPT_GEMM_PAIR 0: 64 or
+                                128 (default)                                 */
   LWE_OPT_GEMM_KCHUNK = 4,   /* K per tensor-core pass: a multiple of 64 up to
                                 the exact bound (2^24-1)/(128 c); 0 = bound   */
-  LWE_OPT_GEMM_PAIR = 5,     /* 1 (default): the GEMM runs on CTA pairs (two
-                                SMs share a 256 x 128 tile, tcgen05
-                                cta_group::2; LWE_OPT_GEMM_BN is then
-                                ignored); 0: one CTA per 128 x BN tile        */
+  LWE_OPT_GEMM_PAIR = 5,     /* 1: the GEMM runs on CTA pairs (two SMs share a
+                                256 x 128 tile, tcgen05 cta_group::2); 0: one
+                                CTA per 128 x BN tile; -1 (default): pairs, or
+                                one CTA per 128 x 64 tile where the product
+                                has at most half as many 256 x 128 tiles as
+                                the GPU has CTA pairs.  LWE_OPT_GEMM_BN is
+                                ignored unless this is 0                      */
   LWE_OPT_SERIAL = 6,        /* 1: work that normally overlaps on the
                                 context's side stream (the tensor path's
                                 limbs, Decaps' H(c)) runs on the caller's

@@ -1031,14 +1031,15 @@ int launch_gemm_sa(const GemmSaArgs &a, int num_sms, cudaStream_t st) {
     // bytes x ncols x K) outgrow a quarter of L2
     if (!b.group_m)
       b.group_m = 4ull * a.ncols * (uint64_t)b.kblocks * BK > (32ull << 20) ? 8u : 1u;
-    // fewer 256 x 128 tiles than half the CTA pairs: 128 x 64 tiles on single
-    // CTAs, four times as many (256 x 4096 at K = 4096: 32 tiles on 76 pairs
-    // against 128 on 152 SMs)
+    // pair < 0: with at most half as many 256 x 128 tiles as CTA pairs, 128 x
+    // 64 tiles on single CTAs, four times as many (256 x 4096 at K = 4096: 32
+    // tiles on 76 pairs against 128 on 152 SMs)
     const uint32_t pair_tiles = ((a.rows + 2 * BM - 1) / (2 * BM)) * ((a.ncols + BN2 - 1) / BN2);
-    const bool pair = a.pair && num_sms >= 2 && 4 * pair_tiles > (uint32_t)num_sms;
-    const int rc = pair                          ? launch_pair(b, num_sms, st)
-                   : (a.pair && num_sms >= 2) || a.bn == 64 ? launch_bn<64>(b, num_sms, st)
-                                          : launch_bn<128>(b, num_sms, st);
+    const bool pair = num_sms >= 2 && (a.pair < 0 ? 4 * pair_tiles > (uint32_t)num_sms : a.pair);
+    const int bn = a.pair < 0 ? 64 : a.bn;
+    const int rc = pair       ? launch_pair(b, num_sms, st)
+                   : bn == 64 ? launch_bn<64>(b, num_sms, st)
+                              : launch_bn<128>(b, num_sms, st);
     if (rc != LWE_OK) return rc;
   }
   return LWE_OK;

@@ -31,8 +31,10 @@ struct GemmSaArgs {
   uint32_t rows;          // 8 * items
   uint32_t logq, B;
   int cmp;                // 0: write out; 1: compare with out
-  int bn;                 // output columns per tile: 64 or 128
-  int pair;               // 1: CTA-pair kernel (256 x 128 tiles, cta_group::2)
+  int bn;                 // output columns per tile where pair is 0: 64 or 128
+  int pair;               // 1: CTA-pair kernel (256 x 128 tiles, cta_group::2);
+                          // 0: single CTAs; -1: pairs, but 128 x 64 tiles on
+                          // single CTAs where pairs would leave SMs idle
   uint32_t group_m;       // tile order: M-blocks per group, M fastest inside
                           // a group (0 or 1: row-major tiles)
   // K-split: this launch contracts K = [k0, k0 + 64 * kblocks) only.  The

@@ -166,7 +166,7 @@ struct lwe_ctx {
   int path = LWE_PATH_AUTO;
   int tensor_min = 64;
   int gemm_bn = 128;
-  int gemm_pair = 1;
+  int gemm_pair = -1;  // LWE_OPT_GEMM_PAIR
   uint32_t gemm_group = 0;  // LWE_OPT_GEMM_GROUP; 0: chosen per launch
   int8_t *ntab = nullptr;    // the sampler table for T (64 KB), built at creation
   uint64_t *tdig = nullptr;  // leaf digests of tree hashes in two launches
@@ -752,7 +752,7 @@ int lwe_ctx_set_option(lwe_ctx *c, int option, int64_t value) {
       c->serial = value != 0;
       return LWE_OK;
     case LWE_OPT_GEMM_PAIR:
-      if (value != 0 && value != 1) return LWE_EINVAL;
+      if (value < -1 || value > 1) return LWE_EINVAL;
       c->gemm_pair = (int)value;
       return LWE_OK;
     case LWE_OPT_PDL:
@@ -1517,7 +1517,7 @@ int pp_encrypt(lwe_pp_ctx *c, const uint32_t *t, const uint32_t *A, uint8_t *ct,
     ga.logq = 16;
     ga.cmp = cmp ? 1 : 0;
     ga.bn = 128;
-    ga.pair = 1;
+    ga.pair = -1;
     ga.clip = c->p.clip;
     ga.kchunk = lwe_gemm_kchunk(c->p.clip);
     ga.partial_out = reinterpret_cast<uint16_t *>(c->partial);

@@ -1,0 +1,76 @@
+"""Which kernels a call launches, read from the CUDA graph that captures it:
+the rules that choose between kernels on size, at both sides of their lines,
+for the number of SMs of the device that runs the test."""
+import ctypes as C
+import re
+
+import pytest
+import torch
+
+from gpu_util import lwe
+
+pytestmark = pytest.mark.gpu
+
+
+class _KernelParams(C.Structure):  # cudaKernelNodeParams
+    _fields_ = [("func", C.c_void_p), ("grid", C.c_uint * 3), ("block", C.c_uint * 3),
+                ("smem", C.c_uint), ("params", C.c_void_p), ("extra", C.c_void_p)]
+
+
+def launches(call):
+    """(mangled kernel name, grid) of every kernel of one call, by capture."""
+    rt = C.CDLL("libcudart.so.13")
+    call()  # lazy set-up happens outside the capture
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(g):
+        call()
+    graph, n = C.c_void_p(g.raw_cuda_graph()), C.c_size_t()
+    assert rt.cudaGraphGetNodes(graph, None, C.byref(n)) == 0
+    nodes = (C.c_void_p * n.value)()
+    assert rt.cudaGraphGetNodes(graph, nodes, C.byref(n)) == 0
+    out = []
+    for node in nodes:
+        kind, p, name = C.c_int(), _KernelParams(), C.c_char_p()
+        assert rt.cudaGraphNodeGetType(C.c_void_p(node), C.byref(kind)) == 0
+        if kind.value == 0:  # cudaGraphNodeTypeKernel
+            assert rt.cudaGraphKernelNodeGetParams(C.c_void_p(node), C.byref(p)) == 0
+            assert rt.cudaFuncGetName(C.byref(name), C.c_void_p(p.func)) == 0
+            out.append((name.value.decode(), tuple(p.grid)))
+    return out
+
+
+def grids(call, kernel):
+    """The grids of the call's launches of `kernel` (any template instance)."""
+    # after the name: template arguments, a namespace's end or a parameter type
+    name_in = re.compile(kernel + r"(?=I|E|\d+[A-Z][a-z])")
+    return [grid for name, grid in launches(call) if name_in.search(name)]
+
+
+def sms():
+    torch.cuda.set_device(0)
+    return torch.cuda.get_device_properties(0).multi_processor_count
+
+
+def matmul_call(n, items, pair):
+    """S A on the tensor cores: 8 items rows."""
+    ctx = lwe.Ctx(lwe.Params(n=n, logq=16, B=2, clip=10, sigma=2.3), max_batch=items)
+    ctx.set_path(lwe.PATH_TENSOR)
+    if pair is not None:
+        ctx.set_option(lwe.OPT_GEMM_PAIR, pair)
+    A = torch.zeros((n, n), dtype=torch.int16, device="cuda")
+    S = torch.zeros((8 * items, n), dtype=torch.int8, device="cuda")
+    out = torch.empty((8 * items, n), dtype=torch.int16, device="cuda")
+    return lambda: lwe.matmul_modq(lwe.SIDE_SA, S, out, n, 16, A=A, ctx=ctx)
+
+
+@pytest.mark.parametrize("pair", [1, 0, -1, None])
+@pytest.mark.parametrize("more", [0, 1])
+def test_gemm_pair_option_selects_the_kernel(pair, more):
+    """1 and 0 hold for every size; -1, the default, takes CTA pairs from more
+    than SMs / 4 tiles of 256 x 128 on (128 columns: one tile per 32 items)."""
+    n, tiles = 128, sms() // 4 + more
+    call = matmul_call(n, 32 * tiles, pair)
+    pairs, singles = len(grids(call, "k_gemm_sa2")), len(grids(call, "k_gemm_sa"))
+    assert pairs + singles == 1
+    assert pairs == (more if pair in (-1, None) else pair)
