@@ -1599,10 +1599,8 @@ void launch_tree(TreeArgs &a, int num_sms, uint32_t warp_max, cudaStream_t st) {
       launch_k(k_tree_roots, (a.count + 5) / 6, 64, 0, st, a);
       return;
     }
-    // up to 8 warps (24 leaves) per CTA, long messages over a cluster of up to 8
-    const uint32_t q = std::max<uint32_t>(1, std::min<uint32_t>(8, (a.m + 23) / 24));
-    const uint32_t w = std::min<uint32_t>((a.m + 3 * q - 1) / (3 * q), TREE_WARP_MAX_THREADS / 32);
-    launch_k_cluster(k_tree_warp, a.count * q, 32 * w, (size_t)a.m * 32, st, q, a);
+    const TreeWarpShape s = tree_warp_shape(a.m);
+    launch_k_cluster(k_tree_warp, a.count * s.ctas, 32 * s.warps, (size_t)a.m * 32, st, s.ctas, a);
     return;
   }
   auto two_launches = [&] {

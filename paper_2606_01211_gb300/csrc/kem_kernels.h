@@ -127,7 +127,18 @@ struct DeriveArgs {
 
 enum { TREE_DIGEST = 0, TREE_ENC_KEY = 1 };
 #define TREE_MAX_THREADS 448  // 14 warps
-#define TREE_WARP_MAX_THREADS 512  // 16 warps, one chunk each
+#define TREE_WARP_MAX_THREADS 512  // 16 warps, three chunks each at a time
+
+// k_tree_warp's CTAs (one cluster) and warps per CTA for a message of m
+// chunks: 24 leaves per CTA, long messages over up to 8
+struct TreeWarpShape {
+  uint32_t ctas, warps;
+};
+inline TreeWarpShape tree_warp_shape(uint32_t m) {
+  const uint32_t q = m <= 24 ? 1u : (m >= 192 ? 8u : (m + 23) / 24);
+  const uint32_t w = (m + 3 * q - 1) / (3 * q);
+  return TreeWarpShape{q, w < TREE_WARP_MAX_THREADS / 32 ? w : TREE_WARP_MAX_THREADS / 32};
+}
 
 // Tree hash of `count` messages of `len` bytes (item e at msgs + e*stride,
 // or msg_ptrs[e]): leaves and root in one kernel, the leaf digests kept in

@@ -515,6 +515,43 @@ int hash_tree(lwe_ctx *c, const uint8_t *msgs, uint64_t stride, uint32_t len, ui
   return check_launch();
 }
 
+// Whether Decaps' H(c), on the other stream, is to have its SMs before the
+// noise takes them.  A noise CTA fills an SM's registers, and programmatic
+// launches let the noise start as soon as the kernels before it have: ahead of
+// H(c), which waits for the end of the previous call, and H(c) then begins when
+// the noise ends.  Its predecessor k_decrypt launched plainly puts H(c) first
+// (8 requests at n = 640 62 -> 44 us; 64 at 8192 373 -> 175; 1 at 4096 88 -> 75).
+// But not where the noise leaves room (an SM for eight of H(c)'s warps), and
+// not where the noise or the product would wait long for it.  With the GEMM
+// that is beyond 15 leaves per SM (200 requests at n = 1344 84 us with the
+// noise first, 93 with the hash; 100 there 77 and 62), but for messages of more
+// than 32 leaves, whose roots are long (90 at 4096 153 and 126), as long as the
+// leaves are not k_tree_leaves_tri's (100 at 6208 199 and 210).  With A stored
+// per item it is beyond 6 leaves per SM (32 at 2048 93 and 103; 20 there 85 and
+// 79), with A regenerated beyond 1 (30 at 640 72 and 77; 10 there 64 and 44).
+bool hash_first(const lwe_ctx *c, uint32_t count, bool tensor, bool fused) {
+  const uint32_t n = c->p.n, len = (uint32_t)ct_bytes(c->p);
+  const uint32_t m = (len + LWE_TREE_CHUNK - 1) / LWE_TREE_CHUNK;
+  const uint64_t sms = (uint64_t)c->num_sms, leaves = (uint64_t)count * m;
+  uint64_t ctas = (uint64_t)count * (2 * ((n + NOISE_RUN_SMALL - 1) / NOISE_RUN_SMALL) + 1);
+  if (ctas > 32 * sms)  // NOISE_RUN, 16 warps to a CTA
+    ctas = ((uint64_t)count * (2 * ((n + NOISE_RUN - 1) / NOISE_RUN) + 1) + 15) / 16;
+  const TreeWarpShape s = tree_warp_shape(m);
+  if ((uint64_t)count * s.ctas <= (sms - std::min(ctas, sms)) * std::max(8 / s.warps, 1u)) return false;
+  if (!tensor) return leaves <= (fused ? sms : 6 * sms);
+  return leaves <= 15 * sms ||
+         (m > 32 && !(m > 96 && count <= tree_warp_max(c->num_sms, len)));
+}
+
+// The first kernel of Decaps' main chain
+void start_decaps(lwe_ctx *c, const DecryptArgs &d, uint32_t count, bool tensor, bool fused,
+                  cudaStream_t st) {
+  const bool pdl = c->pdl;
+  c->pdl = pdl && !hash_first(c, count, tensor, fused);
+  LAUNCH(c, KID_DECRYPT, st, launch_decrypt(d, count, st));
+  c->pdl = pdl;
+}
+
 // Decaps' final key from K', H(c) and the re-encryption flags
 void final_key(lwe_ctx *c, const uint8_t *z, const uint8_t *const *z_ptrs, uint64_t z_off,
                uint32_t count, uint8_t *K, cudaStream_t st) {
@@ -916,8 +953,8 @@ int lwe_decaps(lwe_ctx *c, const uint8_t *sk, const uint16_t *A, const uint8_t *
   }
   tree_hash(c, ct, ctb, (uint32_t)ctb, count, TREE_DIGEST, c->hc, 32, nullptr, 0, ss);
   CUDA_TRY(cudaEventRecord(c->ev_join, ss));
-  DecryptArgs dca = decrypt_args(c, ct, reinterpret_cast<const int8_t *>(sk), nullptr);
-  LAUNCH(c, KID_DECRYPT, st, launch_decrypt(dca, count, st));
+  start_decaps(c, decrypt_args(c, ct, reinterpret_cast<const int8_t *>(sk), nullptr), count, tensor,
+               A == nullptr, st);
   DeriveArgs da = derive_args(c, nullptr, pkh, count);
   da.flags = c->flags;
   LAUNCH(c, KID_DERIVE, st, launch_derive(da, warp_hash_max(c), st));
@@ -983,8 +1020,7 @@ int lwe_decaps_multi(lwe_ctx *c, const uint8_t *const *sk_ptrs, const uint16_t *
   CUDA_TRY(cudaStreamWaitEvent(ss, c->ev_fork, 0));
   tree_hash(c, ct, ctb, (uint32_t)ctb, count, TREE_DIGEST, c->hc, 32, nullptr, 0, ss);
   CUDA_TRY(cudaEventRecord(c->ev_join, ss));
-  DecryptArgs dca = decrypt_args(c, ct, nullptr, sk_ptrs);
-  LAUNCH(c, KID_DECRYPT, st, launch_decrypt(dca, count, st));
+  start_decaps(c, decrypt_args(c, ct, nullptr, sk_ptrs), count, false, A_ptrs == nullptr, st);
   DeriveArgs da = derive_args(c, nullptr, nullptr, count);
   da.flags = c->flags;
   da.pkh_ptrs = sk_ptrs;  // H(pk) is stored inside sk

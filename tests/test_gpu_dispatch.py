@@ -7,7 +7,7 @@ import re
 import pytest
 import torch
 
-from gpu_util import lwe
+from gpu_util import PRESETS, coins, dev, lwe, master_seeds
 
 pytestmark = pytest.mark.gpu
 
@@ -17,8 +17,15 @@ class _KernelParams(C.Structure):  # cudaKernelNodeParams
                 ("smem", C.c_uint), ("params", C.c_void_p), ("extra", C.c_void_p)]
 
 
+class _Edge(C.Structure):  # cudaGraphEdgeData
+    _fields_ = [("from_port", C.c_ubyte), ("to_port", C.c_ubyte), ("type", C.c_ubyte),
+                ("reserved", C.c_ubyte * 5)]
+
+
 def launches(call):
-    """(mangled kernel name, grid) of every kernel of one call, by capture."""
+    """(mangled kernel name, grid, early) of every kernel of one call, by
+    capture; early: it may start before a kernel that it depends on has ended
+    (a programmatic edge)."""
     rt = C.CDLL("libcudart.so.13")
     call()  # lazy set-up happens outside the capture
     torch.cuda.synchronize()
@@ -29,6 +36,12 @@ def launches(call):
     assert rt.cudaGraphGetNodes(graph, None, C.byref(n)) == 0
     nodes = (C.c_void_p * n.value)()
     assert rt.cudaGraphGetNodes(graph, nodes, C.byref(n)) == 0
+    m = C.c_size_t()
+    assert rt.cudaGraphGetEdges(graph, None, None, None, C.byref(m)) == 0
+    tails, heads, data = (C.c_void_p * m.value)(), (C.c_void_p * m.value)(), (_Edge * m.value)()
+    if m.value:
+        assert rt.cudaGraphGetEdges(graph, tails, heads, data, C.byref(m)) == 0
+    early = {heads[i] for i in range(m.value) if data[i].type == 1}  # programmatic
     out = []
     for node in nodes:
         kind, p, name = C.c_int(), _KernelParams(), C.c_char_p()
@@ -36,7 +49,7 @@ def launches(call):
         if kind.value == 0:  # cudaGraphNodeTypeKernel
             assert rt.cudaGraphKernelNodeGetParams(C.c_void_p(node), C.byref(p)) == 0
             assert rt.cudaFuncGetName(C.byref(name), C.c_void_p(p.func)) == 0
-            out.append((name.value.decode(), tuple(p.grid)))
+            out.append((name.value.decode(), tuple(p.grid), node in early))
     return out
 
 
@@ -44,7 +57,7 @@ def grids(call, kernel):
     """The grids of the call's launches of `kernel` (any template instance)."""
     # after the name: template arguments, a namespace's end or a parameter type
     name_in = re.compile(kernel + r"(?=I|E|\d+[A-Z][a-z])")
-    return [grid for name, grid in launches(call) if name_in.search(name)]
+    return [grid for name, grid, _ in launches(call) if name_in.search(name)]
 
 
 def sms():
@@ -74,3 +87,33 @@ def test_gemm_pair_option_selects_the_kernel(pair, more):
     pairs, singles = len(grids(call, "k_gemm_sa2")), len(grids(call, "k_gemm_sa"))
     assert pairs + singles == 1
     assert pairs == (more if pair in (-1, None) else pair)
+
+
+def kem_calls(n, count, path=lwe.PATH_AUTO, stored=True):
+    """Encaps and Decaps of `count` items against a bound key."""
+    ctx = lwe.Ctx(lwe.Params(**dict(PRESETS["P640"], n=n)), max_batch=count)
+    ctx.set_path(path)
+    pk, sk, ct = ctx.empty_pk(1), ctx.empty_sk(1), ctx.empty_ct(count)
+    A = torch.empty((n, n), dtype=torch.int16, device="cuda") if stored else None
+    ctx.keygen(dev(master_seeds(1, seed=n)), pk, sk, A_out=A)
+    ctx.bind_key(pk, sk, A)
+    cs = dev(coins(count, seed=n))
+    K = torch.empty((count, 32), dtype=torch.uint8, device="cuda")
+    return lambda: ctx.encaps(pk, cs, ct, K, A=A), lambda: ctx.decaps(sk, ct, K, A=A)
+
+
+@pytest.mark.parametrize("n,count,stored,first", [
+    (640, 8, True, True), (640, 64, True, True), (8192, 1, True, True), (976, 5, False, True),
+    (640, 1, True, False), (1344, 200, True, False), (640, 30, False, False)])
+def test_decaps_lets_its_hash_start_before_the_noise(n, count, stored, first):
+    """Where the noise would fill every SM and the hash of the ciphertexts, on
+    the other stream, needs few, the main chain's first kernel does not start
+    beside the call before (its followers, and so the noise, may)."""
+    encaps, decaps = kem_calls(n, count, stored=stored)
+
+    def both():
+        encaps()
+        decaps()
+
+    (early,) = [e for name, _, e in launches(both) if "9k_decrypt" in name]
+    assert early != first
