@@ -1607,7 +1607,14 @@ void launch_tree(TreeArgs &a, int num_sms, uint32_t warp_max, cudaStream_t st) {
     // small leaf CTAs when the batch fills the SMs only a few warps deep
     const uint64_t leaves = (uint64_t)a.count * a.m;
     const uint32_t lt = leaves >= (uint64_t)sms * 1024 ? 256u : 64u;
+    // plainly: started beside the last CTAs of the launch before it (the
+    // GEMM's, in Encaps), the leaves crowd on the SMs that come free first,
+    // and the warps of one SM set the time (Encaps of 6000 requests at n =
+    // 208: 365 us, 197 so; 2900 at 1344: 577 and 443)
+    const bool pdl = g_launch_pdl;
+    g_launch_pdl = false;
     launch_k(k_tree_leaves, (uint32_t)((leaves + lt - 1) / lt), lt, 0, st, a);
+    g_launch_pdl = pdl;
     launch_k(k_tree_roots, (a.count + 5) / 6, 64, 0, st, a);
   };
   if (a.m > 32 && dig_fits) {

@@ -117,3 +117,13 @@ def test_decaps_lets_its_hash_start_before_the_noise(n, count, stored, first):
 
     (early,) = [e for name, _, e in launches(both) if "9k_decrypt" in name]
     assert early != first
+
+
+def test_leaf_launch_waits_for_the_kernel_before_it():
+    """The leaves of a batch hashed in two launches are spread evenly over the
+    SMs: the launch does not start beside the GEMM's last CTAs.  The roots do
+    start beside the leaves."""
+    encaps, _ = kem_calls(208, 33 * sms(), path=lwe.PATH_TENSOR)
+    early = {name: e for name, _, e in launches(encaps)}
+    assert [e for name, e in early.items() if "13k_tree_leaves" in name] == [False]
+    assert [e for name, e in early.items() if "12k_tree_roots" in name] == [True]
