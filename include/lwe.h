@@ -156,9 +156,10 @@ enum {
                                 ten threads per Keccak state (lower
                                 latency), larger ones with one state per
                                 thread (higher throughput).  -1 (default):
-                                8 items per SM, tree hashes while there are
-                                at most 44 1024-byte leaves per SM or one
-                                message per SM; 0: always per thread      */
+                                8 items per SM, tree hashes while all their
+                                messages are hashed at once so (a warp per
+                                three 1024-byte leaves, 16 warps per SM);
+                                0: always per thread                      */
   LWE_OPT_PDL = 8,           /* 1 (default): the kernels of Encaps / Decaps
                                 are launched with programmatic stream
                                 serialisation (each may start while the

@@ -228,13 +228,22 @@ uint32_t warp_hash_max(const lwe_ctx *c) {
   return c->tree_warp_max < 0 ? 8u * (uint32_t)c->num_sms : (uint32_t)c->tree_warp_max;
 }
 
-// Tree hashes of m chunks: by default while there are at most 44 leaves per SM
-// (15 warps, one wave of k_tree_warp: 777 messages of 11 chunks, 56 per SM, took
-// 95 us in two waves against 68 with one thread per leaf), and for one short
-// message per SM.
+// Tree hashes of m chunks: by default while the CTAs of k_tree_warp are one
+// wave, i.e. 16 warps per SM (112 registers) in whole CTAs.  On both sides of
+// that, us with it and with one thread per leaf: m = 16 (6 warps) 2 messages
+// per SM 47 and 61, 2.3 84 and 59; m = 7 (3 warps) 4.7 45 and 57, 5.3 70 and
+// 55; m = 65 (3 CTAs of 8) 0.6 80 and 92, 0.7 98 and 94.  Shorter messages, up
+// to 44 leaves and 16 messages per SM: a second wave of small CTAs costs less.
+// (Encaps and Decaps of 1300 requests at n = 64, 83 + 69 us, took 95 + 76
+// without; of 5000 at n = 16, 33 per SM, 188 + 180 with and 198 + 153 without.)
+// Beyond 96 chunks the leaves are a launch of their own: 44 per SM (m = 129: 43
+// 110 and 125, 65 135 and 131), and one message per SM up to 128 chunks.
 uint32_t tree_warp_max(int num_sms, uint32_t len) {
   const uint32_t m = (len + LWE_TREE_CHUNK - 1) / LWE_TREE_CHUNK, sms = (uint32_t)num_sms;
-  return std::max(44u * sms / m, m <= 128 ? sms : 1u);
+  if (m < 7) return std::min(44u * sms / m, 16u * sms);
+  if (m > 96) return std::max(44u * sms / m, m <= 128 ? sms : 1u);
+  const TreeWarpShape s = tree_warp_shape(m);
+  return std::max(sms * (16u / s.warps) / s.ctas, 1u);
 }
 
 struct LaunchScope {

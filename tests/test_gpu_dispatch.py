@@ -127,3 +127,15 @@ def test_leaf_launch_waits_for_the_kernel_before_it():
     early = {name: e for name, _, e in launches(encaps)}
     assert [e for name, e in early.items() if "13k_tree_leaves" in name] == [False]
     assert [e for name, e in early.items() if "12k_tree_roots" in name] == [True]
+
+
+@pytest.mark.parametrize("n,per_sm", [(16, 16), (400, 5), (640, 4), (976, 2), (1344, 2),
+                                      (1600, 1.5), (2000, 1)])
+def test_latency_tree_hash_stays_within_one_wave(n, per_sm):
+    """H(c) runs three Keccak states per warp while its CTAs (or clusters of
+    two, from n = 1600 on) are all resident, and not with one message more (n =
+    16, one leaf each: 16 per SM)."""
+    count = int(per_sm * sms())
+    for items, warp in ((count, 1), (count + 1, 0)):
+        encaps, _ = kem_calls(n, items)
+        assert len(grids(encaps, "k_tree_warp")) == warp, items
