@@ -1617,19 +1617,9 @@ void launch_tree(TreeArgs &a, int num_sms, uint32_t warp_max, cudaStream_t st) {
     g_launch_pdl = pdl;
     launch_k(k_tree_roots, (a.count + 5) / 6, 64, 0, st, a);
   };
-  if (a.m > 32 && dig_fits) {
-    // long messages: every leaf on its own thread, then one warp per root,
-    // once k_tree (below: one thread per message runs its root) would have
-    // root chains of more than 128 chunks (31+ sequential permutations) or
-    // need more than one wave of two CTAs per SM
-    uint32_t t = 1;
-    while (t < a.m && t < 256) t <<= 1;
-    const uint32_t cap = std::max<uint32_t>(
-        1u, std::min<uint32_t>(TREE_MAX_THREADS / t, (48u * 1024u) / (8u * (4 * a.m + 1))));
-    if (a.m > 128 || a.count > 2 * sms * cap) {
-      two_launches();
-      return;
-    }
+  if (a.m > 128 && dig_fits) {  // few messages per CTA: no packing to gain
+    two_launches();
+    return;
   }
   {
     // the balanced schedule of k_tree_bal: leaves of full length filling
@@ -1668,12 +1658,6 @@ void launch_tree(TreeArgs &a, int num_sms, uint32_t warp_max, cudaStream_t st) {
       return;
     }
   }
-  if (a.m >= 2 && dig_fits) {
-    // more leaves than 13 warps per SM (or than 32 messages): Encaps of 4096
-    // requests at n = 1344, 22 leaves each, 826 us with k_tree, 704 so
-    two_launches();
-    return;
-  }
   uint32_t t = 1;
   while (t < a.m && t < 256) t <<= 1;
   a.tpi = t;
@@ -1681,7 +1665,18 @@ void launch_tree(TreeArgs &a, int num_sms, uint32_t warp_max, cudaStream_t st) {
   uint32_t cap = TREE_MAX_THREADS / t;
   cap = std::min<uint32_t>(cap, (48u * 1024u) / (8u * words));
   cap = std::max<uint32_t>(cap, 1u);
-  a.ipc = std::min<uint32_t>(cap, (a.count + sms - 1) / sms);
+  const uint32_t per_sm = (a.count + sms - 1) / sms;
+  if (a.m >= 2 && dig_fits && !(a.m <= 16 && per_sm <= 32 && per_sm <= cap)) {
+    // more leaves than 13 warps per SM (or than 32 messages): two launches
+    // (Encaps of 4096 requests at n = 1344, 22 leaves each, 826 us with
+    // k_tree), but k_tree where it is one wave of up to 14 warps and its roots,
+    // one thread each, are short (at n = 976, 16 leaves, 28 messages per SM:
+    // 442 + 451 us with k_tree, 452 + 490 with two launches; at 29, where
+    // k_tree takes two waves, 626 + 618 against 459 + 499)
+    two_launches();
+    return;
+  }
+  a.ipc = std::min<uint32_t>(cap, per_sm);
   if (a.ipc == 0) a.ipc = 1;
   const uint32_t threads = (a.ipc * t + 31) / 32 * 32;
   const size_t smem = (size_t)a.ipc * words * 8;

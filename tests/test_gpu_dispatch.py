@@ -139,3 +139,11 @@ def test_latency_tree_hash_stays_within_one_wave(n, per_sm):
     for items, warp in ((count, 1), (count + 1, 0)):
         encaps, _ = kem_calls(n, items)
         assert len(grids(encaps, "k_tree_warp")) == warp, items
+
+
+@pytest.mark.parametrize("per_sm,kernel", [(27, "k_tree_bal"), (28, "k_tree"), (29, "k_tree_leaves")])
+def test_tree_schedule_beyond_thirteen_leaf_warps(per_sm, kernel):
+    """At n = 976 (15 full chunks and a short one) 27 messages per SM are 13
+    leaf warps; 28 are one wave of k_tree; 29 are not."""
+    encaps, _ = kem_calls(976, per_sm * sms())
+    assert len(grids(encaps, kernel)) == 1
