@@ -1475,11 +1475,14 @@ void launch_noise(const NoiseArgs &a, int num_sms, cudaStream_t st, bool pp) {
 void launch_mul_as(const MulAsArgs &a, uint32_t count, bool fused, int num_sms, cudaStream_t st) {
   const uint32_t rows = a.rows ? a.rows : a.n, sms = (uint32_t)std::max(num_sms, 1);
   if (!fused) {
-    // 8 warps per 16-row tile, but 4 where 8 (three CTAs per SM) would leave a
-    // short second wave that 4 (six per SM) take along: n = 8192, 512 tiles,
-    // 28.4 us with 8 and 25.7 with 4; n = 16384, 1024 tiles, 95.5 and 101.8
+    // 8 warps per 16-row tile (78 registers: three CTAs per SM), but 4 (94:
+    // five) where those take in one wave what 8 leave a short second wave of.
+    // Back to back, with 8 and with 4: n = 7008 (2.9 tiles per SM) 16.7 and
+    // 18.5 us, 7312 (3.01) 22.7 and 20.6, 8192 27.2 and 23.0, 12160 (5) 51.3
+    // and 45.6, 12176 (5.01) 51.3 and 61.4, 14592 (6) 71.2 and 84.1, 16384 94.2
+    // and 101.7
     const uint64_t tiles = (uint64_t)(rows / 16) * count;
-    if (tiles > 3ull * sms && tiles <= 6ull * sms)
+    if (tiles > 3ull * sms && tiles <= 5ull * sms)
       launch_k(k_mul_as<4>, dim3(rows / 16, count), 128, 0, st, a);
     else
       launch_k(k_mul_as<8>, dim3(rows / 16, count), 256, 0, st, a);

@@ -152,9 +152,9 @@ LWE_DEV void as_flush(int sum[4], float lo[4], float hi[4]) {
 
 // Stored A: a CTA takes a tile of 16 rows, its NW warps split the columns
 // (chunk groups of 4 in turn) with eight 16-byte loads in flight per lane,
-// and their sums meet in shared memory.  Bound by the reads of A: n = 8192,
-// 134 MB from memory, 27.0 us (5.0 TB/s); 16384 100.8 us (5.3 TB/s).  Twelve
-// loads in flight time the same.
+// and their sums meet in shared memory.  Bound by the reads of A: n = 8192
+// 23.0 us back to back, when a part of A is still in L2, 27.0 with L2 flushed
+// (5.0 TB/s); 16384 94.2 us (5.7 TB/s).  Twelve loads in flight time the same.
 template <int NW>
 __global__ void __launch_bounds__(32 * NW) k_mul_as(MulAsArgs a) {
   __shared__ int red[128];

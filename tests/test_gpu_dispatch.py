@@ -147,3 +147,14 @@ def test_tree_schedule_beyond_thirteen_leaf_warps(per_sm, kernel):
     leaf warps; 28 are one wave of k_tree; 29 are not."""
     encaps, _ = kem_calls(976, per_sm * sms())
     assert len(grids(encaps, kernel)) == 1
+
+
+@pytest.mark.parametrize("per_sm,warps", [(3, 8), (3.01, 4), (5, 4), (5.01, 8)])
+def test_stored_AS_takes_four_warps_where_they_are_one_wave(per_sm, warps):
+    """A S with A stored: 16-row tiles per SM on both sides of the lines."""
+    n = 16 * (int(per_sm) * sms() + (per_sm > int(per_sm)))
+    A = torch.zeros((n, n), dtype=torch.int16, device="cuda")
+    St = torch.zeros((8, n), dtype=torch.int8, device="cuda")
+    out = torch.empty((n, 8), dtype=torch.int16, device="cuda")
+    names = [name for name, _, _ in launches(lambda: lwe.matmul_modq(lwe.SIDE_AS, St, out, n, 16, A=A))]
+    assert len(names) == 1 and "8k_mul_asILi%dE" % warps in names[0]

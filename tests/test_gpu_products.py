@@ -71,3 +71,20 @@ def test_products_exact_at_the_largest_sums(n):
     out2 = torch.empty((8, n), dtype=torch.int16, device="cuda")
     lwe.matmul_modq(lwe.SIDE_SA, dev(S), out2, n, 16, A=A_d)
     assert np.array_equal(as_u16(out2), O.mul_SA(S, A, None, 16))
+
+
+@pytest.mark.parametrize("n", [7312, 8192])
+def test_stored_AS_of_one_wave_matches_exact_sums(n):
+    """The 4-warp instance of the stored A S (more than three 16-row tiles
+    per SM), whose column stride of 128 chunks n = 7312 is no multiple of:
+    against whole-number sums in 64-bit floating point."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n)
+    A = torch.randint(0, 65536, (n, n), generator=g, device="cuda", dtype=torch.int32).to(torch.int16)
+    St = torch.randint(-128, 128, (8, n), generator=g, device="cuda", dtype=torch.int8)
+    E = torch.randint(-128, 128, (n, 8), generator=g, device="cuda", dtype=torch.int8)
+    out = torch.empty((n, 8), dtype=torch.int16, device="cuda")
+    lwe.matmul_modq(lwe.SIDE_AS, St, out, n, 16, A=A, E=E)
+    exact = (A.to(torch.int32) & 0xFFFF).to(torch.float64) @ St.to(torch.float64).T
+    exact = (exact.to(torch.int64) + E.long()) & 0xFFFF
+    assert np.array_equal(as_u16(out).astype(np.int64), host(exact))
