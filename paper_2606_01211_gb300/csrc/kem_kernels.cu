@@ -1493,15 +1493,20 @@ void launch_mul_as(const MulAsArgs &a, uint32_t count, bool fused, int num_sms, 
     launch_k(k_mul_as_gen, sms, 512, AS_GEN_SMEM, st, a, count);
     return;
   }
-  // clusters of R CTAs walk the 16-row tiles of each item
-  const uint32_t tiles = rows / 16, groups = (a.n / 8 + 3) / 4;  // groups of 4 chunks per tile
+  // Clusters of R CTAs walk the 16-row tiles of each item.  A tile's time goes
+  // by its groups of 4 chunks, one per warp of the cluster and step; a cluster's
+  // barriers cost about as much as one more step.  With 1, 2 and 4 CTAs: n =
+  // 1344 12.5, 18.5, 20.6 us; 3600 43.1, 41.1, 59.4; 5008 79.9, 77.9, 98.4; 6208
+  // 97.1, 111, 123; 8192 156, 152, 187; 16384 524, 553, 626.
+  const uint32_t tiles = rows / 16, groups = (a.n / 8 + 3) / 4;
   uint32_t best_R = 1, best_G = 1;
   uint64_t best_cost = ~0ull;
   for (uint32_t R = 1; R <= 8; R++) {
     const uint32_t slots = std::max(R, cluster_slots(R, sms));
     const uint32_t G = std::min(tiles, std::max<uint32_t>(1u, slots / (R * count)));
     const uint64_t ctas = (uint64_t)R * G * count;
-    const uint64_t cost = ((ctas + slots - 1) / slots) * ((tiles + G - 1) / G) * ((groups + R - 1) / R + 3);
+    const uint64_t rounds = ((ctas + slots - 1) / slots) * ((tiles + G - 1) / G);
+    const uint64_t cost = rounds * (groups + (R > 1 ? 15 * R : 0)) * 840 / R;
     if (cost < best_cost) {
       best_cost = cost;
       best_R = R;

@@ -158,3 +158,18 @@ def test_stored_AS_takes_four_warps_where_they_are_one_wave(per_sm, warps):
     out = torch.empty((n, 8), dtype=torch.int16, device="cuda")
     names = [name for name, _, _ in launches(lambda: lwe.matmul_modq(lwe.SIDE_AS, St, out, n, 16, A=A))]
     assert len(names) == 1 and "8k_mul_asILi%dE" % warps in names[0]
+
+
+@pytest.mark.parametrize("n", [1344, 1600, 6208, 7200])
+def test_regenerated_AS_split_counts_the_barriers(n):
+    """One item's A S with A regenerated: one CTA per 16-row tile where that
+    fills the rounds of the SMs well, not clusters whose barriers cost more
+    than the even split gains (on 152 SMs)."""
+    if sms() != 152:
+        pytest.skip("sizes chosen for 152 SMs")
+    seed = torch.zeros(16, dtype=torch.uint8, device="cuda")
+    St = torch.zeros((8, n), dtype=torch.int8, device="cuda")
+    out = torch.empty((n, 8), dtype=torch.int16, device="cuda")
+    (grid,) = grids(lambda: lwe.matmul_modq(lwe.SIDE_AS, St, out, n, 16, seedA=seed),
+                    "k_mul_as_gen_split")
+    assert grid == (1, min(n // 16, sms()), 1)
