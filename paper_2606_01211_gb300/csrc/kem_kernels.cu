@@ -1362,16 +1362,20 @@ cudaError_t lwe_upload_aes_table(const uint32_t T0[256]) {
   return cudaMemcpyToSymbol(g_aes_img, img.data(), AES_TABLE_WORDS * sizeof(uint32_t));
 }
 
-// CTAs of the AES product kernels (one per SM) that run at once in clusters
-// of R, per device: clusters do not straddle GPCs, so on a 152-SM GB300 not
-// every R uses every SM.  Filled by lwe_kernel_smem_setup.
-static uint32_t g_cluster_slots[128][9];
+// CTAs that run at once in clusters of R, per device: of the AES product
+// kernels (one per SM) and of k_sa (two).  Clusters do not straddle GPCs, so on
+// a 152-SM GB300 not every R uses every SM: 152, 152, 138, 144, 140, 138, 105,
+// 120 for R = 1 .. 8, and 304, 304, 291, 296, 290, 276, 266, 288 of k_sa.
+// Filled by lwe_kernel_smem_setup.
+static uint32_t g_cluster_slots[128][9], g_sa_slots[128][9];
 
-static uint32_t cluster_slots(uint32_t R, uint32_t sms) {
+// the current device's row of a table
+static const uint32_t *device_slots(const uint32_t (*table)[9]) {
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 128) return sms / R * R;
-  const uint32_t n = g_cluster_slots[dev][R];
-  return n ? n : sms / R * R;
+  return cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 128 ? table[dev] : nullptr;
+}
+static uint32_t cluster_slots(const uint32_t *row, uint32_t R, uint32_t per_sm, uint32_t sms) {
+  return std::max(R, row && row[R] ? row[R] : per_sm * sms / R * R);
 }
 
 static cudaError_t query_cluster_slots() {
@@ -1394,6 +1398,11 @@ static cudaError_t query_cluster_slots() {
     e = cudaOccupancyMaxActiveClusters(&n, k_sa_gen<false>, &cfg);
     if (e != cudaSuccess) return e;
     g_cluster_slots[dev][R] = (uint32_t)n * R;
+    cfg.blockDim = dim3(256, 1, 1);
+    cfg.dynamicSmemBytes = 0;
+    e = cudaOccupancyMaxActiveClusters(&n, k_sa<false>, &cfg);
+    if (e != cudaSuccess) return e;
+    g_sa_slots[dev][R] = (uint32_t)n * R;
   }
   return cudaSuccess;
 }
@@ -1402,10 +1411,11 @@ static cudaError_t query_cluster_slots() {
 // of `work` units so that the last wave wastes least; every CTA has a fixed
 // cost of `fixed` units.
 static uint32_t best_split(uint64_t tiles, uint32_t work, uint32_t fixed, uint32_t sms) {
+  const uint32_t *row = device_slots(g_cluster_slots);
   uint32_t best = 1;
   uint64_t best_cost = ~0ull;
   for (uint32_t R = 1; R <= 8 && R <= work; R++) {
-    const uint32_t slots = std::max(R, cluster_slots(R, sms));
+    const uint32_t slots = cluster_slots(row, R, 1, sms);
     const uint64_t waves = (tiles * R + slots - 1) / slots;
     const uint64_t cost = waves * ((work + R - 1) / R + fixed);
     if (cost < best_cost) {
@@ -1499,10 +1509,11 @@ void launch_mul_as(const MulAsArgs &a, uint32_t count, bool fused, int num_sms, 
   // 1344 12.5, 18.5, 20.6 us; 3600 43.1, 41.1, 59.4; 5008 79.9, 77.9, 98.4; 6208
   // 97.1, 111, 123; 8192 156, 152, 187; 16384 524, 553, 626.
   const uint32_t tiles = rows / 16, groups = (a.n / 8 + 3) / 4;
+  const uint32_t *row = device_slots(g_cluster_slots);
   uint32_t best_R = 1, best_G = 1;
   uint64_t best_cost = ~0ull;
   for (uint32_t R = 1; R <= 8; R++) {
-    const uint32_t slots = std::max(R, cluster_slots(R, sms));
+    const uint32_t slots = cluster_slots(row, R, 1, sms);
     const uint32_t G = std::min(tiles, std::max<uint32_t>(1u, slots / (R * count)));
     const uint64_t ctas = (uint64_t)R * G * count;
     const uint64_t rounds = ((ctas + slots - 1) / slots) * ((tiles + G - 1) / G);
@@ -1528,17 +1539,21 @@ void launch_mul_sa(const MulSaArgs &a, uint32_t items, bool fused, bool cmp, int
   if (fused) {
     R = best_split((uint64_t)cbs * items, steps, 14, sms);
   } else {
-    // column groups per CTA and row split: few waves of two CTAs per SM (90
-    // registers), counting 64 steps for a CTA's start and end, and two row
-    // steps per warp at least; of equals the narrowest, whose clusters are
-    // small.  A from memory, n = 8192: 256 CTAs as 1 x 2, 2 x 4 or 4 x 8 take
-    // 31.3, 32.6 and 33.2 us, 384 as 1 x 3 43.6; n = 12000: 282 as 2 x 3 59.9,
-    // 4 x 6 106 (clusters of 6 do not fill the GPCs); 16384: 1 x 1 100.7
-    const uint32_t slots = 2 * sms;
+    // column groups per CTA and row split: few waves of the CTAs that run at
+    // once (two per SM at 88 registers, less what clusters leave), counting 64
+    // steps for a CTA's start and end, and two row steps per warp at least; of
+    // equals the narrowest, whose clusters are small.  A from memory, n = 8192:
+    // 256 CTAs as 1 x 2, 2 x 4 or 4 x 8 take 28.6, 30.8 and 30.8 us, 384 as 1 x
+    // 3 38.8; n = 16384, two items: 2 x 1 171, 4 x 7 227.
+    // Small calls: n = 976, 10 items, 160 CTAs as 1 x 1 9.9 us, 280 as 4 x 7,
+    // more than the 266 that run at once, 16.5; 640, 20 items, 1 x 1 9.1, 300 as
+    // 2 x 3 13.9
+    const uint32_t *row = device_slots(g_sa_slots);
     uint64_t best_cost = ~0ull;
     R = 1;
     for (uint32_t g = 1; g <= 4; g *= 2)
       for (uint32_t r = 1; r <= 8 && (r == 1 || steps * g >= 16 * r); r++) {
+        const uint64_t slots = cluster_slots(row, r, 2, sms);
         const uint64_t ctas = (uint64_t)((a.n + 64 * g - 1) / (64 * g)) * items * r;
         const uint64_t cost = (ctas + slots - 1) / slots * ((uint64_t)steps * g / r + 64);
         if (cost < best_cost) {

@@ -173,3 +173,17 @@ def test_regenerated_AS_split_counts_the_barriers(n):
     (grid,) = grids(lambda: lwe.matmul_modq(lwe.SIDE_AS, St, out, n, 16, seedA=seed),
                     "k_mul_as_gen_split")
     assert grid == (1, min(n // 16, sms()), 1)
+
+
+@pytest.mark.parametrize("n,items", [(640, 20), (976, 5), (976, 10), (1344, 10), (2048, 5), (16384, 2)])
+def test_stored_SA_split_fits_the_clusters_that_run_at_once(n, items):
+    """S' A with A stored, a few items: the split does not count on CTAs that
+    its clusters leave no room for (a seventh of the SMs for clusters of 7)."""
+    if sms() != 152:
+        pytest.skip("clusters counted on 152 SMs")
+    A = torch.zeros((n, n), dtype=torch.int16, device="cuda")
+    S = torch.zeros((8 * items, n), dtype=torch.int8, device="cuda")
+    out = torch.empty((8 * items, n), dtype=torch.int16, device="cuda")
+    (grid,) = grids(lambda: lwe.matmul_modq(lwe.SIDE_SA, S, out, n, 16, A=A), "k_sa")
+    room = {2: 304, 3: 291, 4: 296, 5: 290, 6: 276, 7: 266, 8: 288}
+    assert grid[1] == 1 or grid[0] * grid[1] * grid[2] <= room[grid[1]]
