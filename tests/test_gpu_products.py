@@ -9,6 +9,7 @@ import pytest
 import torch
 
 from gpu_util import O, as_u16, dev, host, lwe, master_seeds, params
+from test_gpu_dispatch import grids
 
 pytestmark = pytest.mark.gpu
 
@@ -88,3 +89,31 @@ def test_stored_AS_of_one_wave_matches_exact_sums(n):
     exact = (A.to(torch.int32) & 0xFFFF).to(torch.float64) @ St.to(torch.float64).T
     exact = (exact.to(torch.int64) + E.long()) & 0xFFFF
     assert np.array_equal(as_u16(out).astype(np.int64), host(exact))
+
+
+@pytest.mark.parametrize("n", [16, 304])
+def test_items_beyond_the_tables_a_cta_holds_match_oracle(n):
+    """KeyGen of so many items that a warp takes whole row tiles (at least 32
+    per SM).  n = 16, one tile each: a CTA's range spans 33 or 34 items, nine
+    rounds of the four keys whose tables it holds; n = 304, 19 tiles: ranges
+    begin inside an item.  The items at both sides of the CTAs' and of the
+    rounds' boundaries."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    tiles = n // 16
+    count = -(-33 * sms // tiles) + 7
+    p, po = params("P640", n=n)
+    ctx = lwe.Ctx(p, max_batch=count)
+    ms = master_seeds(count, seed=n + 1)
+    seeds, pk, sk = dev(ms), ctx.empty_pk(count), ctx.empty_sk(count)
+    ctx.keygen(seeds, pk, sk)
+    assert len(grids(lambda: ctx.keygen(seeds, pk, sk), "k_mul_as_gen")) == 1
+    pk_h, sk_h = host(pk), host(sk)
+    units, check = count * tiles, {0, count - 1}
+    for b in (0, 1, 2, sms // 2, sms - 1):
+        first, last = units * b // sms // tiles, (units * (b + 1) // sms - 1) // tiles
+        check |= {i for i in range(first - 1, first + 10)} | {last - 1, last, last + 1}
+    for i in sorted(i for i in check if 0 <= i < count):
+        pk_o, sk_o = O.keygen(po, bytes(ms[i]))
+        assert np.array_equal(pk_h[i], pk_o), i
+        assert np.array_equal(sk_h[i], sk_o), i
+    ctx.close()
