@@ -247,7 +247,7 @@ def cpu_large_n(threads: int, batch: int = 1024):
 
 def per_request_rate(kem, lwe, torch, stream, pairs: int = 2048):
     """The plain per-request GPU path: one P976 Encaps and then its Decaps
-    per call (count = 1, CUDA-core kernels, the key bound as in the batched
+    per call (count = 1, per-item kernels, the key bound as in the batched
     step), back to back on one stream, host wall-clock from the first launch
     to the final synchronisation; the coins are the batched step's, and the
     keys are checked identical to the batched step's."""
@@ -590,7 +590,7 @@ def run_ours(args, rank, world, local_rank):
     energy = energy_measure(kem, torch, stream, local_rank) if extras and not args.no_energy else None
 
     # the same 4096-item step with direct launches (no graph) on the
-    # CUDA-core product instead of the tensor cores (still one batched call
+    # per-item product instead of the tensor cores (still one batched call
     # per operation)
     def direct_rate(path):
         kem.ctx.set_path(path)
@@ -618,7 +618,7 @@ def run_ours(args, rank, world, local_rank):
         torch.cuda.synchronize()
         rate, same, m = per_request_rate(kem, lwe, torch, stream)
         per_req = {"value": rate, "unit": UNIT, "pairs": m, "identical_to_batched": same,
-                   "how": "one Encaps and its Decaps per call (count = 1, CUDA-core path), "
+                   "how": "one Encaps and its Decaps per call (count = 1, per-item path), "
                           "back to back on one stream, host wall-clock"}
     kem.close()
 
@@ -929,7 +929,7 @@ def paper_profile(lwe, torch, dev, cpu: bool = True,
 def large_n(lwe, torch, dev, batch: int = 1024, names=("P16384", "P32768")):
     """n = 16384 and 32768 (A = 0.5 / 2 GiB): one KeyGen, Encaps and Decaps
     per call with A stored in HBM vs regenerated tile by tile inside the
-    kernels (CUDA-core path), and Encaps of `batch` items against one key
+    kernels (per-item path), and Encaps of `batch` items against one key
     on the tensor path (K split into exact passes).  CUDA-event ms per call
     (median of 3); the batched figure also as Encaps/s."""
     stream = torch.cuda.current_stream()

@@ -123,7 +123,7 @@ int lwe_ctx_destroy(lwe_ctx *ctx);
 /* Product path for Encrypt's S' A (Alg. 2): */
 enum {
   LWE_PATH_AUTO = 0,   /* tensor path when count >= the tuned threshold  */
-  LWE_PATH_SKINNY = 1, /* per-item CUDA-core kernels ("plain" path)      */
+  LWE_PATH_SKINNY = 1, /* per-item kernels on mma.sync ("plain" path)    */
   LWE_PATH_TENSOR = 2  /* stacked S' as one exact two-limb bf16 tcgen05
                           GEMM (tensor cores, fp32 accumulation; K split
                           into passes of at most (2^24-1)/(128 c) columns).
@@ -159,12 +159,16 @@ enum {
                                 8 items per SM, tree hashes while all their
                                 messages are hashed at once so (a warp per
                                 three 1024-byte leaves, 16 warps per SM);
-                                0: always per thread                      */
+                                0: per thread in every launch, but for the
+                                roots of batched tree hashes, which run so
+                                whatever the value                        */
   LWE_OPT_PDL = 8,           /* 1 (default): the kernels of Encaps / Decaps
                                 are launched with programmatic stream
                                 serialisation (each may start while the
                                 previous one drains, and waits on the
-                                device for its results); 0: plain launches */
+                                device for its results), but for a few
+                                that an early start slows down; 0: plain
+                                launches                                   */
   LWE_OPT_GEMM_GROUP = 9     /* tensor-core GEMM tile order: the persistent
                                 CTAs visit output tiles in groups of this
                                 many row blocks of S' (the row block varies
@@ -225,7 +229,7 @@ int lwe_decaps(lwe_ctx *ctx, const uint8_t *sk, const uint16_t *A,
  *               either all-stored or all-regenerated.
  * coins / ct / K are laid out as in lwe_encaps / lwe_decaps.  Results are
  * identical to one single-key call per item.  These calls always take the
- * CUDA-core product (the tensor path needs one shared A).  Pointer arrays
+ * per-item product (the tensor path needs one shared A).  Pointer arrays
  * must be 8-byte aligned, key objects 16-byte aligned. */
 int lwe_encaps_multi(lwe_ctx *ctx, const uint8_t *const *pk_ptrs,
                      const uint8_t *const *pkh_ptrs, const uint16_t *const *A_ptrs,
@@ -278,7 +282,7 @@ int lwe_expand_A(const uint8_t *seedA, uint32_t n, uint32_t logq,
  * (and its n equals n and its max_batch covers k/8), SA may take the
  * tensor-core path and its workspace -- then every |S| must be at most the
  * context's clip, which bounds the exact K per tensor-core pass; otherwise
- * the CUDA-core kernels run. */
+ * the per-item kernels run. */
 enum { LWE_SIDE_AS = 0, LWE_SIDE_SA = 1 };
 int lwe_matmul_modq(lwe_ctx *ctx, int side, const uint16_t *A,
                     const uint8_t *seedA, const int8_t *S, uint32_t n,
@@ -302,7 +306,7 @@ int lwe_matmul_modq(lwe_ctx *ctx, int side, const uint16_t *A,
  * A_rows [row1 - row0][n] uint16: the block of rows (row row0 first), or
  * NULL to regenerate those rows from seedA [16] (device).  S as in
  * lwe_matmul_modq (S^T [8][n] for AS, S [k][n] for SA, full width).  row0
- * and row1 multiples of 16 with row0 < row1 <= n.  CUDA-core kernels;
+ * and row1 multiples of 16 with row0 < row1 <= n.  Per-item kernels;
  * needs no context.  LWE_EINVAL for bad sizes or pointers. */
 int lwe_matmul_modq_rows(int side, const uint16_t *A_rows, const uint8_t *seedA,
                          const int8_t *S, uint32_t n, uint32_t k, uint32_t logq,
@@ -316,7 +320,7 @@ int lwe_matmul_modq_rows(int side, const uint16_t *A_rows, const uint8_t *seedA,
 #define LWE_NOALLOC_SCRATCH_BYTES (1024u * 1024u)
 
 /* Encaps exactly as lwe_encaps (same inputs, outputs, layouts and results;
- * CUDA-core path), for callers that cannot allocate device memory and so
+ * per-item path), for callers that cannot allocate device memory and so
  * cannot create an lwe_ctx: code that must not call cudaMalloc/cudaFree
  * because the host application owns every device allocation through its own
  * pool, or because a request path cannot afford an allocation's implicit

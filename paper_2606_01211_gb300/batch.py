@@ -13,7 +13,7 @@ per-bit encryptions of one Encaps into one launch, Sec. 3.2).
 
 autotune() times the candidate GEMM kernels (CTA pairs on 256 x 128 tiles,
 or one CTA on 128 x 64 / 128 x 128 tiles) and the items-per-call threshold
-above which the tensor path beats the CUDA-core path, for a given (n,
+above which the tensor path beats the per-item path, for a given (n,
 batch), and caches the choice in a JSON file.
 """
 from __future__ import annotations

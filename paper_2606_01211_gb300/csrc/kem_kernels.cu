@@ -90,13 +90,14 @@ __global__ void __launch_bounds__(512, 1) k_expand_A(const uint8_t *__restrict__
 }
 
 // ---------------------------------------------------------------------------
-// Noise: a warp generates one run of NOISE_RUN counter blocks of one stream
-// of one item (4 blocks per lane, two at a time, contiguous stores).
-// Sampling (Tab. 1, rounded Gaussian by CDF inversion): a 16-bit word w gives
-// t = w >> 1, |e| = #{i : t > T[i]}, e < 0 iff w & 1.  Every CTA first
-// tabulates e for all 65536 words in shared memory (64 KB of int8), so a
-// sample costs one byte load; the table is built from T with the same
-// comparison rule.
+// Noise: a warp generates one run of counter blocks of one stream of one item
+// (4 blocks per lane, two at a time, in batches; one in small calls; contiguous
+// stores).  Sampling (Tab. 1, rounded Gaussian by CDF inversion): a 16-bit word
+// w gives t = w >> 1, |e| = #{i : t > T[i]}, e < 0 iff w & 1.  A table of e for
+// all 65536 words (64 KB of int8) sits in shared memory, so a sample costs one
+// byte load; it is made from T with the same comparison rule when the context
+// is created and copied in by each CTA, or made by the CTA where there is no
+// context.
 // ---------------------------------------------------------------------------
 #define NOISE_TAB_OFF AES_SMEM_BYTES
 #define NOISE_SMEM_BYTES (AES_SMEM_BYTES + 65536)
@@ -781,9 +782,10 @@ LWE_DEV void tree_tri_out(const TreeArgs &a, uint32_t e, bool in, const KeccakTr
 // Named barriers (fixed thread counts, every warp meets each of its
 // barriers exactly once): 1 leaf warps of SMSPs 1-3 -> warp 13 (320);
 // 2 warps 0, 4 -> helper 14 (96); 4 warps 8, 12 -> helper 15 (96);
-// 3 helpers and warp 13 -> the eleven root warps (448).  At most 96 registers per thread (no spills):
-// a CTA then leaves room in the SM's register file for the CTAs of Decaps'
-// small kernels, which run beside its H(c) on the other stream.
+// 3 helpers and warp 13 -> the eleven root warps (448).  At most 96 registers
+// per thread (20 bytes of spill stores, 44 of loads; k_tree_dense 16 and 12): a
+// CTA then leaves room in the SM's register file for the CTAs of Decaps' small
+// kernels, which run beside its H(c) on the other stream.
 #define TB_SPLIT 6
 #define TB_SLOTS 128
 
@@ -1016,16 +1018,15 @@ __global__ void __maxnreg__(112) k_tree_warp(TreeArgs a) {
   tree_tri_out(a, e, km.grp == 0, km, lane, s);
 }
 
-// Tree hash of long messages (more than 32 chunks: ciphertexts and public
-// keys of n >= 4096) in two launches.  k_tree_leaves hashes every 1024-byte
-// chunk of the batch on its own thread (message e's chunk c on thread
-// e m + c, all SMs busy whatever the batch size) and writes the digests to
-// a.dig ([count][m][4] words); k_tree_roots then runs each message's root,
-// a sequential sponge over 32 m bytes, on one warp with the state spread
-// over the lanes, which shortens that chain about twofold against one
-// thread (and, for Encaps, derives the key).  k_tree instead gave each such
-// message a group of up to 256 threads and ran the root on one thread while
-// the group waited.
+// Tree hash in two launches: long messages, and batches beyond what one CTA per
+// SM packs.  k_tree_leaves hashes every 1024-byte chunk of the batch on its own
+// thread (message e's chunk c on thread e m + c, all SMs busy whatever the
+// batch size) and writes the digests to a.dig ([count][m][4] words);
+// k_tree_roots then runs the roots, sequential sponges over 32 m bytes, three
+// per warp with ten threads each (keccak_warp.cuh), which takes 2.3 us a
+// permutation against one thread's 4.7-5.6, and for Encaps derives the keys.
+// k_tree gives each message a group of up to 256 threads and runs the root on
+// one thread while the group waits.
 __global__ void __launch_bounds__(256) k_tree_leaves(TreeArgs a) {
   pdl_trigger();
   pdl_wait();
@@ -1607,9 +1608,11 @@ void launch_derive(const DeriveArgs &a, uint32_t warp_max, cudaStream_t st) {
   launch_k(k_derive, (a.count + 31) / 32, 64, 0, st, a);
 }
 
-// One CTA per SM where the batch allows (the leaf work is one wave: CTAs of
-// equal size spread it evenly), at most TREE_MAX_THREADS threads and 48 KB
-// of digests per CTA.
+// Few messages: three Keccak states per warp.  Else one state per thread, one
+// CTA per SM where the batch allows (the leaf work is one wave: CTAs of equal
+// size spread it evenly): k_tree_bal and k_tree_dense, then k_tree for one wave
+// of short messages or without a digest buffer (at most TREE_MAX_THREADS
+// threads and 48 KB of digests per CTA); two launches for the rest.
 void launch_tree(TreeArgs &a, int num_sms, uint32_t warp_max, cudaStream_t st) {
   a.m = (a.len + LWE_TREE_CHUNK - 1) / LWE_TREE_CHUNK;
   const uint32_t sms = num_sms > 0 ? (uint32_t)num_sms : 1u;

@@ -19,7 +19,8 @@ enum { NOISE_I8 = 0, NOISE_BF16 = 1, NOISE_BOTH = 2, NOISE_UNIFORM = 3 };
 // fill the SMs' warps use runs of NOISE_RUN_SMALL, dealt out over the SMs.
 #define NOISE_RUN 128
 #define NOISE_RUN_SMALL 32
-static_assert(256 % NOISE_RUN == 0, "a noise run lies inside one 256-block counter window");
+static_assert(256 % NOISE_RUN == 0 && 256 % NOISE_RUN_SMALL == 0,
+              "a noise run lies inside one 256-block counter window");
 
 struct NoiseOut {
   void *base;            // item e writes at base + e * item_stride (bytes)
@@ -188,7 +189,7 @@ void launch_mul_as(const MulAsArgs &a, uint32_t count, bool fused, int num_sms, 
 void launch_decrypt(const DecryptArgs &a, uint32_t count, cudaStream_t st);
 void launch_mul_sa(const MulSaArgs &a, uint32_t items, bool fused, bool cmp, int num_sms,
                    cudaStream_t st);
-// launches of at most warp_max items hash with one Keccak state per warp
+// launches of at most warp_max items hash with ten threads per Keccak state
 void launch_keygen_seeds(const KeygenSeedArgs &a, uint32_t warp_max, cudaStream_t st);
 void launch_derive(const DeriveArgs &a, uint32_t warp_max, cudaStream_t st);
 void launch_tree(TreeArgs &a, int num_sms, uint32_t warp_max, cudaStream_t st);

@@ -173,7 +173,7 @@ struct lwe_ctx {
   uint64_t tdig_words = 0;
   bool serial = false;  // LWE_OPT_SERIAL: side-stream work on the caller's stream
   bool pdl = true;      // LWE_OPT_PDL
-  int64_t tree_warp_max = -1;  // LWE_OPT_WARP_HASH_MAX; -1: the number of SMs
+  int64_t tree_warp_max = -1;  // LWE_OPT_WARP_HASH_MAX; -1: warp_hash_max, tree_warp_max
   bool timing = false;
   uint64_t launches = 0;
   std::vector<TimedLaunch> pending;

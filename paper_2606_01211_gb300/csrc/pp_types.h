@@ -14,7 +14,7 @@ struct ModQ {
 enum { PP_BINOMIAL = 0, PP_GAUSS = 1 };
 
 struct PpNoiseOut {
-  void *out;       // int8 (binomial, Gaussian) or int32 (uniform) samples
+  void *out;       // int8 samples
   uint32_t count;  // samples
   uint32_t kind;
   uint32_t domain;
