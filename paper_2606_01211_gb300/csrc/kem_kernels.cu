@@ -1505,10 +1505,12 @@ void launch_mul_as(const MulAsArgs &a, uint32_t count, bool fused, int num_sms, 
     return;
   }
   // Clusters of R CTAs walk the 16-row tiles of each item.  A tile's time goes
-  // by its groups of 4 chunks, one per warp of the cluster and step; a cluster's
-  // barriers cost about as much as one more step.  With 1, 2 and 4 CTAs: n =
-  // 1344 12.5, 18.5, 20.6 us; 3600 43.1, 41.1, 59.4; 5008 79.9, 77.9, 98.4; 6208
-  // 97.1, 111, 123; 8192 156, 152, 187; 16384 524, 553, 626.
+  // by its groups of 4 chunks, 16 per CTA and step; a cluster's barriers cost
+  // about as much as one more step, the last tile's less.  With 1, 2 and 4 CTAs:
+  // n = 1344 12.5, 18.5, 20.6 us; 3600 43.1, 41.1, 59.4; 5008 79.9, 77.9, 98.4;
+  // 6208 97.1, 111, 123; 8192 156, 152, 187; 16384 524, 553, 626.  One round:
+  // KeyGen, Encaps and Decaps at n = 640 with 1, 2 and 3 178.9, 176.1, 174.1,
+  // at n = 976 193.9, 187.5, 194.6 (two rounds with 3).
   const uint32_t tiles = rows / 16, groups = (a.n / 8 + 3) / 4;
   const uint32_t *row = device_slots(g_cluster_slots);
   uint32_t best_R = 1, best_G = 1;
@@ -1518,7 +1520,7 @@ void launch_mul_as(const MulAsArgs &a, uint32_t count, bool fused, int num_sms, 
     const uint32_t G = std::min(tiles, std::max<uint32_t>(1u, slots / (R * count)));
     const uint64_t ctas = (uint64_t)R * G * count;
     const uint64_t rounds = ((ctas + slots - 1) / slots) * ((tiles + G - 1) / G);
-    const uint64_t cost = rounds * (groups + (R > 1 ? 15 * R : 0)) * 840 / R;
+    const uint64_t cost = rounds * groups * 840 / R + (R > 1 ? (15 * rounds - 6) * 840 : 0);
     if (cost < best_cost) {
       best_cost = cost;
       best_R = R;
