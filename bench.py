@@ -355,12 +355,12 @@ def algorithmic(p, count):
 CSRC = os.path.join(ROOT, "paper_2606_01211_gb300", "csrc")
 TRAFFIC = {
     # kernel: (bytes per step, launches per step, [(file, function or None)], fingerprint, profile)
-    "k_tree": (129.379584e6, 2,
+    "k_tree": (129.320448e6, 2,
                [("kem_kernels.cu", "k_tree_bal"), ("kem_kernels.cu", "launch_tree"),
                 ("kem_kernels.cu", "tree_tri_out"), ("keccak.cuh", None),
                 ("keccak_warp.cuh", None)],
-               "761cb1539b8e7e03", "profiles/k_tree_p976.md"),
-    "k_gemm_tc": (295.791104e6, 2, [("gemm_tc.cu", None)], "a11460dc8c0e227f",
+               "a4da1c89f2235e3c", "profiles/k_tree_p976.md"),
+    "k_gemm_tc": (296.145408e6, 2, [("gemm_tc.cu", None)], "ff9300a61b8088d7",
                   "profiles/k_gemm_sa2_p976.md"),
     "k_noise": (69.633280e6, 2,
                 [("kem_kernels.cu", "k_noise"), ("kem_kernels.cu", "noise_runs"),
