@@ -57,3 +57,28 @@ def test_batch_schedules_agree_with_it(n, count):
     assert np.array_equal(keys[0], keys[1])
     assert ctx.device_error() == 0
     ctx.close()
+
+
+def test_one_wave_of_k_tree_agrees_with_it():
+    """28 messages of 16 chunks per SM, more leaves than the packed schedules
+    take (k_tree, its last CTA ragged): Encaps' keys and Decaps' equal those of
+    one message per CTA."""
+    torch.cuda.set_device(0)
+    count = 28 * torch.cuda.get_device_properties(0).multi_processor_count - 5
+    p, _ = params("P976")
+    ctx = lwe.Ctx(p, max_batch=count)
+    pk, sk = ctx.empty_pk(1), ctx.empty_sk(1)
+    ctx.keygen(dev(master_seeds(1, seed=28)), pk, sk)
+    coins = dev(np.random.default_rng(28).integers(0, 256, (count, 32), dtype=np.uint8))
+    ct = ctx.empty_ct(count)
+    keys = []
+    for warp_max in (-1, count):
+        K, K2 = (torch.empty((count, 32), dtype=torch.uint8, device="cuda") for _ in range(2))
+        ctx.set_option(lwe.OPT_WARP_HASH_MAX, warp_max)
+        ctx.encaps(pk, coins, ct, K)
+        ctx.decaps(sk, ct, K2)
+        keys += [host(K), host(K2)]
+    for k in keys[1:]:
+        assert np.array_equal(keys[0], k)
+    assert ctx.device_error() == 0
+    ctx.close()
